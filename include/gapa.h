@@ -353,8 +353,7 @@ int gapa_set_fitness_kernel(gapa_ctx* ctx, int variant);
  * adjacency matrix (Eqs. 14-17), N = gapa_set_sixdst_hops (default 6):
  * with rowsum(v) = the live nodes within N hops of live v (itself included),
  * PC_N = (Σ_live rowsum - live) / 2 and MCN_N = max_live rowsum, equal to PC
- * and MCN once N reaches every component's diameter; node genes, n <= 8192,
- * tensor-core products.  Applies to gapa_fitness and the generation and run
+ * and MCN once N reaches every component's diameter; node genes, n <= 8192.  Applies to gapa_fitness and the generation and run
  * calls (batches take PC and MCN); gapa_fitness_noalloc computes PC. */
 #define GAPA_OBJECTIVE_PC 0
 #define GAPA_OBJECTIVE_MCN 1
@@ -362,19 +361,23 @@ int gapa_set_fitness_kernel(gapa_ctx* ctx, int variant);
 #define GAPA_OBJECTIVE_SIXDST_MCN 3
 int gapa_set_objective(gapa_ctx* ctx, int objective);
 int gapa_set_sixdst_hops(gapa_ctx* ctx, int hops);
-/* Tensor-core path of the SixDST products (identical results): TMA (the
- * default: tcgen05.mma with the accumulator in tensor memory, operands loaded
- * by cp.async.bulk.tensor from a tensor map by a producer thread while another
- * issues the products, six stages, 256 x 256 output tiles when the padded size
+/* Path of the SixDST objectives (identical results): TMA (tcgen05.mma with the
+ * accumulator in tensor memory, operands loaded by cp.async.bulk.tensor from a
+ * tensor map by a producer thread while another issues the products, six stages, 256 x 256 output tiles when the padded size
  * is a multiple of 256, else as TCGEN05), TCGEN05 (the same products with
  * operands loaded by every thread with cp.async, three stages; 256 x 256 tiles
  * when the padded size allows, else 128 x 128), TCGEN05_128 (128 x 128 tiles
  * only) or MMA_SYNC (warp-level mma.sync).  A device-side wait that runs out is
- * reported as GAPA_ERR_TIMEOUT. */
+ * reported as GAPA_ERR_TIMEOUT.  BITS forms the same matrix hop by hop from bit
+ * rows along the arcs of the sparse graph, without products.  AUTO (the
+ * default) takes BITS where N hops cost less than the products, else the best
+ * product available. */
 #define GAPA_SIXDST_MMA_SYNC 0
 #define GAPA_SIXDST_TCGEN05 1
 #define GAPA_SIXDST_TCGEN05_128 2
 #define GAPA_SIXDST_TMA 3
+#define GAPA_SIXDST_AUTO 4
+#define GAPA_SIXDST_BITS 5
 int gapa_set_sixdst_kernel(gapa_ctx* ctx, int kernel);
 
 /* Failure-path check of the device-side bounded waits (the paper has no

@@ -57,6 +57,9 @@ void free_graph(DeviceGraph& g) {
     cudaFree(g.lo_ptr);
     cudaFree(g.lo_col);
     cudaFree(g.palt);
+    cudaFree(g.sb_rank);
+    cudaFree(g.sb_line);
+    cudaFree(g.sb_col);
     for (SparseForest& f : g.spf) {
         void* tabs[] = {f.kids, f.croot, f.csize, f.sub, f.bysize, f.cost};
         for (void* q : tabs) cudaFree(q);
@@ -1072,6 +1075,13 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
             return frc;
         }
     }
+    if (n <= kBitsMaxNodes) {
+        const int brc = gapa_sixdst_bits_upload(g, rp, sorted);
+        if (brc != GAPA_OK) {
+            free_graph(g);
+            return brc;
+        }
+    }
     c->g = g;
     return GAPA_OK;
 }
@@ -1332,13 +1342,17 @@ int gapa_read_bandwidth(gapa_ctx* c, int64_t bytes, int32_t reps, double* gbs) {
 int gapa_set_sixdst_kernel(gapa_ctx* c, int kernel) {
     if (!c) return gapa_fail(GAPA_ERR_INVALID_ARG, "ctx is NULL");
     if (kernel != GAPA_SIXDST_MMA_SYNC && kernel != GAPA_SIXDST_TCGEN05 && kernel != GAPA_SIXDST_TCGEN05_128 &&
-        kernel != GAPA_SIXDST_TMA)
+        kernel != GAPA_SIXDST_TMA && kernel != GAPA_SIXDST_AUTO && kernel != GAPA_SIXDST_BITS)
         return gapa_fail(GAPA_ERR_INVALID_ARG, "unknown SixDST kernel %d", kernel);
+    if (kernel == GAPA_SIXDST_AUTO || kernel == GAPA_SIXDST_BITS) {
+        c->sixdst_route = kernel;
+        return GAPA_OK;
+    }
     if (kernel != GAPA_SIXDST_MMA_SYNC && !c->sixdst_t5_ok)
         return gapa_fail(GAPA_ERR_INVALID_ARG, "the tcgen05 product does not fit in this device's shared memory");
     if (kernel == GAPA_SIXDST_TMA && !c->sixdst_t7_ok)
         return gapa_fail(GAPA_ERR_INVALID_ARG, "the TMA product is not available on this device");
-    c->sixdst_kernel = kernel;
+    c->sixdst_route = kernel;
     return GAPA_OK;
 }
 

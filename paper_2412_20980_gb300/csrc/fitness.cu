@@ -734,6 +734,10 @@ static bool sparse_selected(const gapa_ctx* c) {
 }
 
 int gapa_fitness_prepare(gapa_ctx* c, int s) {
+    if (c->objective == GAPA_OBJECTIVE_SIXDST_PC || c->objective == GAPA_OBJECTIVE_SIXDST_MCN) {
+        const int rc = gapa_sixdst_prepare(c, s);
+        if (rc != GAPA_OK) return rc;
+    }
     const size_t lab_bytes = (size_t)c->g.n * 4;
     const bool tree = c->fitness_variant != GAPA_FITNESS_EDGES && c->fitness_variant != GAPA_FITNESS_SAMPLED;
     if (sparse_selected(c)) {

@@ -200,7 +200,14 @@ struct DeviceGraph {
     SparseForest spf[kSpForests];
     int sp_nforests = 0;
     int sp_hub[2] = {-1, -1};
+    // SixDST by bit rows (n <= kBitsMaxNodes): adjacency by degree rank (sixdst_bits.cu)
+    int* sb_rank = nullptr;             // [n] original id -> rank
+    int* sb_line = nullptr;             // [sb_hubs + sb_slices + 1] first line of 32 entries
+    unsigned short* sb_col = nullptr;
+    int sb_hubs = 0, sb_slices = 0;
 };
+
+constexpr int kBitsMaxNodes = 8192;  // the SixDST objectives' size limit
 
 constexpr int kProbe = 8;
 constexpr int kOrderCap = 1 << 16;  // members ordered by cost per fitness launch (larger batches: in order)
@@ -243,13 +250,12 @@ struct gapa_ctx {
     int objective = 0;        // GAPA_OBJECTIVE_PC or GAPA_OBJECTIVE_MCN
     int genes = 0;            // GAPA_GENES_NODES or GAPA_GENES_EDGES
     int sixdst_hops = 6;      // N of the SixDST objectives
-    int sixdst_kernel = 0;    // SixDST products: 0 = mma.sync, 1 = tcgen05 (256-wide tiles where the padded size
-                              // allows), 2 = tcgen05 with 128-wide tiles only, 3 = tcgen05 with TMA loads and
-                              // split roles (the default when it fits; 256-wide tiles, else as 1)
     bool sixdst_t5_ok = false;  // the tcgen05 product's shared memory fits on this device
     bool sixdst_t6_ok = false;  // and so does the 256-wide tile's
     bool sixdst_t7_ok = false;  // and the TMA kernel's (with the driver's tensor-map encoder)
-    void* sdst_buf = nullptr;  // SixDST matrices and deletion bitmaps of a member batch
+    int sixdst_route = GAPA_SIXDST_AUTO;  // GAPA_SIXDST_AUTO, GAPA_SIXDST_BITS, or a dense product
+    size_t sdst_bits_smem_max = 0;  // max dynamic shared memory of the bit-row kernel
+    void* sdst_buf = nullptr;  // SixDST matrices and deletion bitmaps of a member batch, or the bit-row kernel's sums
     size_t sdst_cap = 0;
     // (mu+lambda) and roulette scratch
     int32_t* kids = nullptr;
@@ -387,6 +393,15 @@ int gapa_launch_fitness_ig(gapa_ctx* c, const int32_t* pop, int s, int k, int64_
 int gapa_launch_fitness_sixdst(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
                                int* kernels = nullptr);
 int gapa_sixdst_init(gapa_ctx* c);
+int gapa_sixdst_prepare(gapa_ctx* c, int s);  // scratch for s members (outside any capture)
+// SixDST by bit rows (sixdst_bits.cu): set-up, whether the graph's rows fit, the adjacency by rank
+// (at upload), its scratch for s members and its launch.
+int gapa_sixdst_bits_init(gapa_ctx* c);
+bool gapa_sixdst_bits_fits(const gapa_ctx* c);
+int gapa_sixdst_bits_upload(DeviceGraph& g, const std::vector<int32_t>& rp, const std::vector<int32_t>& col);
+int gapa_sixdst_bits_prepare(gapa_ctx* c, int s);
+int gapa_launch_sixdst_bits(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
+                            int* kernels);
 int gapa_launch_selftest_wait(gapa_ctx* c, long long limit, cudaStream_t st);
 int gapa_launch_read_probe(const void* buf, size_t bytes, int passes, int grid, unsigned* sink, cudaStream_t st);
 int gapa_ig_prepare(gapa_ctx* c, int s);

@@ -869,11 +869,12 @@ int gapa_launch_selftest_wait(gapa_ctx* c, long long limit, cudaStream_t st) {
 }
 
 int gapa_sixdst_init(gapa_ctx* c) {
+    const int brc = gapa_sixdst_bits_init(c);
+    if (brc != GAPA_OK) return brc;
     const int bytes = 2 * kT5Stages * kT5StageBytes;
     if ((size_t)bytes + 1024 > c->smem_optin) return GAPA_OK;  // the tcgen05 product stays unavailable
     GAPA_CUDA(cudaFuncSetAttribute(sdst_gemm_t5_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     c->sixdst_t5_ok = true;
-    c->sixdst_kernel = 1;
     if ((size_t)kT6Smem + 1024 <= c->smem_optin) {
         GAPA_CUDA(cudaFuncSetAttribute(sdst_gemm_t6_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kT6Smem));
         c->sixdst_t6_ok = true;
@@ -881,9 +882,49 @@ int gapa_sixdst_init(gapa_ctx* c) {
     if ((size_t)kT7Smem + 1024 <= c->smem_optin && t7_encoder()) {
         GAPA_CUDA(cudaFuncSetAttribute(sdst_gemm_t7_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kT7Smem));
         c->sixdst_t7_ok = true;
-        c->sixdst_kernel = GAPA_SIXDST_TMA;
     }
     return GAPA_OK;
+}
+
+// The dense product: the chosen one, else the best this device has.
+static int dense_kernel(const gapa_ctx* c) {
+    if (c->sixdst_route <= GAPA_SIXDST_TMA) return c->sixdst_route;
+    return c->sixdst_t7_ok ? GAPA_SIXDST_TMA : c->sixdst_t5_ok ? GAPA_SIXDST_TCGEN05 : GAPA_SIXDST_MMA_SYNC;
+}
+
+// AUTO: bit rows where N hops along the arcs cost less than the dense products.  Bit rows handle at
+// least 2.0e12 words/s of the (2E + n) n / 32 per hop and member (1.9e12 at n = 1000 and mean degree 2.7,
+// 4.3e12 at n = 2018 and degree 32), with no credit for stopping early; the dense path takes its
+// products' n^3 at 2.0e15 (256-wide TMA tiles) or 0.7e15 multiply-adds/s, 0.34 ps per matrix byte to
+// build and one pass over a matrix at 7.9 GB/s per member's CTA at the end.  Measured with 80 members and
+// 6 hops, bits / dense: n = 1000: 30 / 443 us at degree 2.7, 105 / 446 at 32, 430 / 451 at 128; n = 2018:
+// 90 / 1702, 465 / 1719, 2016 / 1727; n = 7500 (16 members): 333 / 52,900 and 8,900 / 52,900 at 128.
+static bool bits_selected(const gapa_ctx* c, int s) {
+    if (c->sixdst_route == GAPA_SIXDST_BITS) return true;
+    if (c->sixdst_route != GAPA_SIXDST_AUTO || !gapa_sixdst_bits_fits(c)) return false;
+    const double n = c->g.n, np = (c->g.n + kPad - 1) / kPad * kPad;
+    int products = -1;
+    for (int e = c->sixdst_hops; e > 0; e >>= 1) products += (e & 1) + (e > 1);
+    const double rate = dense_kernel(c) == GAPA_SIXDST_TMA && (int)np % 256 == 0 ? 2.0e15 : 0.7e15;
+    const double bits = s * (double)c->sixdst_hops * (2.0 * c->g.num_edges + n) * n / 32 / 2.0e12;
+    const double dense = s * (products * np * np * np / rate + np * np * 0.34e-12) + np * np / 7.9e9;
+    return bits <= dense;
+}
+
+// Members per batch of the dense path (three matrices each, within 2 GiB) and its scratch.
+static int dense_batch(int n, int s) {
+    const size_t np = (size_t)(n + kPad - 1) / kPad * kPad;
+    return (int)std::min<size_t>(std::max<size_t>(1, ((size_t)2 << 30) / (3 * np * np)), (size_t)std::max(s, 1));
+}
+
+static int dense_reserve(gapa_ctx* c, int batch) {
+    const size_t np = (size_t)(c->g.n + kPad - 1) / kPad * kPad;
+    return gapa_reserve(&c->sdst_buf, &c->sdst_cap, (size_t)batch * (3 * np * np + (np + 31) / 32 * 4), 1);
+}
+
+int gapa_sixdst_prepare(gapa_ctx* c, int s) {
+    if (c->g.n > kBitsMaxNodes) return GAPA_OK;  // the launch reports it
+    return bits_selected(c, s) ? gapa_sixdst_bits_prepare(c, s) : dense_reserve(c, dense_batch(c->g.n, s));
 }
 
 int gapa_launch_fitness_sixdst(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
@@ -892,12 +933,11 @@ int gapa_launch_fitness_sixdst(gapa_ctx* c, const int32_t* pop, int s, int k, in
     const int np = (n + kPad - 1) / kPad * kPad;
     if (np > 8192) return gapa_fail(GAPA_ERR_INVALID_ARG, "SixDST fitness needs n <= 8192 (n = %d)", n);
     const int hops = c->sixdst_hops;
+    if (bits_selected(c, s)) return gapa_launch_sixdst_bits(c, pop, s, k, fit, st, kernels);
     const size_t mat = (size_t)np * np;
     const int words = (np + 31) / 32;
-    // members per batch: three matrices each, within 2 GiB
-    int batch = (int)std::max<size_t>(1, ((size_t)2 << 30) / (3 * mat));
-    batch = std::min(batch, std::max(s, 1));
-    int rc = gapa_reserve(&c->sdst_buf, &c->sdst_cap, (size_t)batch * 3 * mat + (size_t)batch * words * 4, 1);
+    const int batch = dense_batch(n, s);
+    int rc = dense_reserve(c, batch);
     if (rc != GAPA_OK) return rc;
     unsigned char* buf[3];
     for (int i = 0; i < 3; ++i) buf[i] = reinterpret_cast<unsigned char*>(c->sdst_buf) + (size_t)i * batch * mat;
@@ -912,10 +952,11 @@ int gapa_launch_fitness_sixdst(gapa_ctx* c, const int32_t* pop, int s, int k, in
         int base = 0, res = -1;
         const int tiles = np / kTile;
         const dim3 grid(tiles * (tiles + 1) / 2, bm);
-        const bool t5 = c->sixdst_kernel >= 1;
+        const int kernel = dense_kernel(c);
+        const bool t5 = kernel >= 1;
         // 256-wide tiles where the padded size allows them; TMA loads with split roles by default
-        const bool t7 = c->sixdst_kernel == GAPA_SIXDST_TMA && c->sixdst_t7_ok && np % kT6Tile == 0;
-        const bool t6 = (c->sixdst_kernel == 1 || (c->sixdst_kernel == GAPA_SIXDST_TMA && !t7)) && c->sixdst_t6_ok &&
+        const bool t7 = kernel == GAPA_SIXDST_TMA && c->sixdst_t7_ok && np % kT6Tile == 0;
+        const bool t6 = (kernel == 1 || (kernel == GAPA_SIXDST_TMA && !t7)) && c->sixdst_t6_ok &&
                         np % kT6Tile == 0;
         const int tiles6 = np / kT6Tile;
         const dim3 grid6(tiles6 * (tiles6 + 1) / 2, bm);

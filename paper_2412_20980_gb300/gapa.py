@@ -431,8 +431,9 @@ class Context:
         return float(out.value)
 
     def set_sixdst_kernel(self, kernel: int):
-        """SixDST products (same results): 3 tcgen05 with TMA loads and split roles (the default where
-        available), 1 tcgen05 with cp.async loads, 2 tcgen05 with 128-wide tiles only, 0 mma.sync."""
+        """SixDST path (same results): 4 automatic (the default), 5 bit rows along the arcs, 3 tcgen05
+        products with TMA loads and split roles, 1 tcgen05 with cp.async loads, 2 tcgen05 with 128-wide
+        tiles only, 0 mma.sync."""
         _check(self.lib.gapa_set_sixdst_kernel(self.handle, kernel))
 
     def set_sixdst_hops(self, hops: int):
