@@ -159,27 +159,42 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(GemmArgs a) {
 // Residual degrees of each row's deletion set D: among the live nodes with a
 // neighbour in D, r0 counts those with no live neighbour left and r1 those
 // with exactly one; r2 counts the two-node components of G[V\D] adjacent to
-// D.  Every (gene v, neighbour u) pair with u live scans N(u) until a second
-// live neighbour shows up; u is counted by the first deleted node of its
-// adjacency list, so exactly once.  A pendant u whose live neighbour w has no
-// other live neighbour closes a two-node component, counted at u when u < w
-// or when w has no deleted neighbour (degree 1), so once.  The deletion bitmap sits in
-// shared memory (ceil(n/32) words); one CTA per row.  A warp takes 32 genes
-// at a time: the (gene, neighbour) pairs of the genes of degree below 32 are
-// laid end to end and dealt out one per lane (a lane finds its gene by binary
-// search over the warp's degree prefix sums), and the whole warp walks each
-// larger adjacency together.  Genes outside [0, n) are ignored.
+// D.  One CTA per row, bitmaps of ceil(n/32) words in shared memory.  A warp
+// takes 32 genes at a time: the arcs of the genes of degree below 32 are laid
+// end to end and dealt out one per lane (the genes that start within the 32
+// arcs of a step as one bit mask: a lane's gene is a population count away),
+// and the whole warp walks each larger adjacency together.  Genes outside
+// [0, n) are ignored.
+//
+// A node of degree d has at most one live neighbour only when at least d - 1 arcs
+// of D reach it: twice at least when d > 2.  So every arc's head sets its bit in
+// a `once` bitmap (set beforehand for nodes of degree one and two), a head found
+// set there goes on to a `twice` bitmap, and the live nodes of that one are
+// listed and examined with all lanes at the end: one shared-memory atomic
+// settles most arcs.  A pendant u whose live neighbour w has no other live
+// neighbour closes a two-node component, counted at u when u < w or when w has
+// no deleted neighbour (degree 1), so once.
+//
+// Bound by instruction issue.  Measured (2048 rows of 2000 genes, n = 100000,
+// mean degree 6): 143 us.  A gather of the head's entry of the
+// neighbour table per arc took 274 us with two neighbours per entry and 222 us with
+// four (bound by the L1's 32 tag lookups per gather), and stays where three
+// bitmaps exceed shared memory; the bitmaps with a binary search per arc and a
+// list appended to arc by arc 158 us.
 __device__ __forceinline__ bool bm_dead(const unsigned* bm, int w) { return (bm[w >> 5] >> (w & 31)) & 1u; }
 
-// Per node: {first arc, degree, a, b}: a and b are the two neighbours of lowest
-// degree (earlier arcs first among equals; -1 when absent).  Any two live
-// neighbours settle a node, and a deletion set that favours hubs is least likely
-// to hold u's lowest-degree neighbours.  One thread per node, once per surrogate.
+// Per node: its four neighbours of lowest degree (earlier arcs first among equals; -1 when absent).  Any
+// two live neighbours settle a node, and a deletion set that favours hubs is least likely to hold its
+// lowest-degree neighbours; a node of degree four or less (the sign bit of the last one) is settled by
+// its entry whatever it holds.
+// With two neighbours beside the node's arc range (the same 16 bytes) 36 % of the pairs of random sets
+// still scanned an adjacency, since the deleted node itself is often one of the two.  One thread per
+// node, once per surrogate.
 __global__ void nbr_table_kernel(const int* __restrict__ row_ptr, const int* __restrict__ col, int n,
                                  int4* __restrict__ T) {
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
         const int b = row_ptr[u], d = row_ptr[u + 1] - b;
-        int a1 = -1, a2 = -1, d1 = INT_MAX, d2 = INT_MAX;
+        int a[4] = {-1, -1, -1, -1}, da[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX};
         for (int q0 = b; q0 < b + d; q0 += 4) {
             int x[4], dx[4];
 #pragma unroll
@@ -188,37 +203,58 @@ __global__ void nbr_table_kernel(const int* __restrict__ row_ptr, const int* __r
             for (int i = 0; i < 4; ++i) dx[i] = x[i] >= 0 ? __ldg(row_ptr + x[i] + 1) - __ldg(row_ptr + x[i]) : INT_MAX;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (x[i] < 0) continue;
-                if (dx[i] < d1) {
-                    a2 = a1;
-                    d2 = d1;
-                    a1 = x[i];
-                    d1 = dx[i];
-                } else if (dx[i] < d2) {
-                    a2 = x[i];
-                    d2 = dx[i];
+                int xi = x[i], di = dx[i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {  // insert before the first entry of larger degree
+                    if (di < da[j]) {
+                        const int ta = a[j], td = da[j];
+                        a[j] = xi;
+                        da[j] = di;
+                        xi = ta;
+                        di = td;
+                    }
                 }
             }
         }
-        T[u] = make_int4(b, d, a1, a2);
+        T[u] = make_int4(a[0], a[1], a[2], d <= 4 ? a[3] | INT_MIN : a[3]);
     }
 }
 
-// Live neighbours of u, counted up to two (the last one seen in *w).
-__device__ __forceinline__ int live_upto2(const unsigned* bm, const int4* __restrict__ T, const int* __restrict__ col,
-                                          int u, int* first_dead, int* w) {
+// Live neighbours of u, counted up to two; with fewer than two, *first_dead is the lowest deleted
+// neighbour (adjacencies are ascending; -1 if none) and *w the live one.
+__device__ __forceinline__ int live_upto2(const unsigned* bm, const int4* __restrict__ T,
+                                          const int* __restrict__ row_ptr, const int* __restrict__ col, int u,
+                                          int* first_dead, int* w) {
     const int4 tu = __ldg(T + u);
-    if (tu.w >= 0 && !bm_dead(bm, tu.z) && !bm_dead(bm, tu.w)) return 2;
-    int live = 0;
-    for (int q = tu.x; q < tu.x + tu.y; ++q) {
-        const int x = __ldg(col + q);
-        if (bm_dead(bm, x)) {
-            if (first_dead && *first_dead < 0) *first_dead = x;
+    const int x[4] = {tu.x, tu.y, tu.z, tu.w == -1 ? -1 : tu.w & INT_MAX};
+    int live = 0, fd = INT_MAX, lw = -1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (x[i] < 0) continue;
+        if (bm_dead(bm, x[i])) {
+            fd = min(fd, x[i]);
         } else {
-            *w = x;
-            if (++live >= 2) return 2;
+            lw = x[i];
+            ++live;
         }
     }
+    if (live >= 2) return 2;
+    if (tu.w >= 0) {  // a longer adjacency may hold more
+        const int e = __ldg(row_ptr + u + 1);
+        live = 0;
+        fd = INT_MAX;
+        for (int q = __ldg(row_ptr + u); q < e; ++q) {
+            const int y = __ldg(col + q);
+            if (bm_dead(bm, y)) {
+                fd = min(fd, y);
+            } else {
+                lw = y;
+                if (++live >= 2) return 2;
+            }
+        }
+    }
+    *first_dead = fd == INT_MAX ? -1 : fd;
+    *w = lw;
     return live;
 }
 
@@ -230,41 +266,84 @@ struct __align__(16) ResidRow {
     float4 z;
 };
 
-// (u live) -> +1 to c0 or c1 when u has at most one live neighbour and v is its
-// first deleted one; +1 to c2 when that neighbour closes a two-node component.
-// Most live u keep the two neighbours of their table entry: one 16-byte read settles them.
-__device__ __forceinline__ void resid_pair(const unsigned* bm, const int4* __restrict__ T,
-                                           const int* __restrict__ col, int v, int u, int& c0, int& c1, int& c2) {
-    if (bm_dead(bm, u)) return;
+// Live u with a deleted neighbour -> +1 to c0 or c1 when it has at most one live neighbour; +1 to c2 when
+// that neighbour closes a two-node component.  v >= 0: only if v is u's first deleted neighbour (the
+// caller examines u once per deleted neighbour).  times: how often u's first deleted neighbour is counted.
+template <class Times>
+__device__ __forceinline__ void resid_node(const unsigned* bm, const int4* __restrict__ T,
+                                           const int* __restrict__ row_ptr, const int* __restrict__ col, int v, int u,
+                                           int& c0, int& c1, int& c2, const Times& times) {
     int first_dead = -1, w = -1;
-    const int live = live_upto2(bm, T, col, u, &first_dead, &w);
-    if (live >= 2 || first_dead != v) return;
-    c0 += live == 0;
-    if (live == 1) {
-        c1 += 1;
-        int wl = -1;
-        const int4 tw = __ldg(T + w);
-        if ((u < w || tw.y == 1) && live_upto2(bm, T, col, w, nullptr, &wl) == 1) c2 += 1;
+    const int live = live_upto2(bm, T, row_ptr, col, u, &first_dead, &w);
+    if (live >= 2 || (v >= 0 && first_dead != v)) return;
+    const int add = times(first_dead);
+    if (live == 0) {
+        c0 += add;
+        return;
+    }
+    c1 += add;
+    int wd = -1, wl = -1;
+    // w's own neighbour u is live: a deleted neighbour of w is there unless w's degree is 1
+    if (live_upto2(bm, T, row_ptr, col, w, &wd, &wl) == 1 && (u < w || wd < 0)) c2 += add;
+}
+
+constexpr int kResidList = 1024;  // nodes listed at a time
+
+// Bit u set: node u has degree one or two.
+__global__ void low_degree_kernel(const int* __restrict__ row_ptr, int n, unsigned* __restrict__ low) {
+    for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < (n + 31) / 32; w += gridDim.x * blockDim.x) {
+        unsigned bits = 0;
+        for (int i = 0; i < 32 && 32 * w + i < n; ++i) {
+            const int d = row_ptr[32 * w + i + 1] - row_ptr[32 * w + i];
+            if (d == 1 || d == 2) bits |= 1u << i;
+        }
+        low[w] = bits;
     }
 }
 
-__global__ void __launch_bounds__(256) resid_kernel(const int* __restrict__ pop, int rows, int k, int n,
-                                                    const int4* __restrict__ T, const int* __restrict__ col,
-                                                    ResidRow* __restrict__ out) {
+// sums: the running sums of the three counts and of their squares (exact integers, so the order does not
+// matter) and the rows done, all zero at launch.  The last row to finish turns them into the means and
+// standard deviations (FP64 with explicit rounding: mean = S1 / rows, var = S2 / rows - mean^2, sd =
+// max(sqrt(var), 1); ms[0..2] = means, ms[3..5] = deviations) and zeroes them for the next launch.
+template <bool kOnce>
+__global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop, int rows, int k, int n,
+                                                     const unsigned* __restrict__ low,
+                                                     const int4* __restrict__ T, const int* __restrict__ row_ptr,
+                                                     const int* __restrict__ col, ResidRow* __restrict__ out,
+                                                     unsigned long long* __restrict__ sums, double* __restrict__ ms) {
     extern __shared__ unsigned bm[];
-    __shared__ int red[3][8];
+    __shared__ int red[3][32];
+    __shared__ bool s_last;
+    __shared__ int s_list[kOnce ? kResidList : 1], s_count;
+    __shared__ int2 s_own[32][32];  // per warp: of the genes with dealt arcs, first arc less prefix, and the gene
     const int r = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (r >= rows) return;
     const int words = (n + 31) >> 5;
-    for (int w = t; w < words; w += blockDim.x) bm[w] = 0u;
-    __syncthreads();
-    const int* genes = pop + (size_t)r * k;
-    for (int j = t; j < k; j += blockDim.x) {
-        const int v = genes[j];
-        if (v >= 0 && v < n) atomicOr(&bm[v >> 5], 1u << (v & 31));
+    unsigned *once = bm + words, *twice = once + words;
+    for (int w = t; w < words; w += blockDim.x) {
+        bm[w] = 0u;
+        if (kOnce) {
+            once[w] = __ldg(&low[w]);
+            twice[w] = 0u;
+        }
     }
     __syncthreads();
+    const int* genes = pop + (size_t)r * k;
+    bool repeated = false;
+    for (int j = t; j < k; j += blockDim.x) {
+        const int v = genes[j];
+        if (v >= 0 && v < n) repeated |= (atomicOr(&bm[v >> 5], 1u << (v & 31)) >> (v & 31)) & 1u;
+    }
+    repeated = __syncthreads_or(repeated);
     int c0 = 0, c1 = 0, c2 = 0;
+    auto arc = [&](int v, int u) {
+        if (!kOnce) {
+            if (!bm_dead(bm, u)) resid_node(bm, T, row_ptr, col, v, u, c0, c1, c2, [](int) { return 1; });
+            return;
+        }
+        const unsigned bit = 1u << (u & 31);
+        if (atomicOr(&once[u >> 5], bit) & bit) atomicOr(&twice[u >> 5], bit);
+    };
     const int nwarps = blockDim.x >> 5;
     for (int j0 = warp * 32; j0 < k; j0 += nwarps * 32) {
         const int j = j0 + lane;
@@ -272,12 +351,11 @@ __global__ void __launch_bounds__(256) resid_kernel(const int* __restrict__ pop,
         if (v >= n) v = -1;
         int b = 0, e = 0;
         if (v >= 0) {
-            const int4 tv = __ldg(T + v);
-            b = tv.x;
-            e = tv.x + tv.y;
+            b = __ldg(row_ptr + v);
+            e = __ldg(row_ptr + v + 1);
         }
         const bool big = e - b >= 32;
-        // small adjacencies: flatten the pairs over the lanes
+        // small adjacencies: deal the arcs out over the lanes
         const int d = big ? 0 : e - b;
         int incl = d;
 #pragma unroll
@@ -285,20 +363,21 @@ __global__ void __launch_bounds__(256) resid_kernel(const int* __restrict__ pop,
             const int x = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += x;
         }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        const int total = __shfl_sync(0xffffffffu, incl, 31), start = incl - d;
+        const unsigned dealt = __ballot_sync(0xffffffffu, d > 0);
+        __syncwarp();
+        if (d > 0) s_own[warp][__popc(dealt & ((1u << lane) - 1))] = make_int2(b - start, v);
+        __syncwarp();
+        int before = 0;  // genes that start in earlier steps
         for (int base = 0; base < total; base += 32) {
+            const unsigned at = (unsigned)(start - base);
+            const unsigned starts = __reduce_or_sync(0xffffffffu, d > 0 && at < 32u ? 1u << at : 0u);
             const int idx = base + lane;
-            // owner = the first lane whose inclusive prefix exceeds idx
-            int lo = 0, hi = 31;
-#pragma unroll
-            for (int step = 0; step < 5; ++step) {
-                const int mid = (lo + hi) >> 1;
-                const int pm = __shfl_sync(0xffffffffu, incl, mid);
-                if (pm > idx) hi = mid; else lo = mid + 1;
+            if (idx < total) {
+                const int2 own = s_own[warp][before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
+                arc(own.y, __ldg(col + own.x + idx));
             }
-            const int ov = __shfl_sync(0xffffffffu, v, lo), ob = __shfl_sync(0xffffffffu, b, lo),
-                      oi = __shfl_sync(0xffffffffu, incl, lo), od = __shfl_sync(0xffffffffu, d, lo);
-            if (idx < total) resid_pair(bm, T, col, ov, __ldg(col + ob + (idx - (oi - od))), c0, c1, c2);
+            before += __popc(starts);
         }
         unsigned many = __ballot_sync(0xffffffffu, big);
         while (many) {
@@ -306,8 +385,46 @@ __global__ void __launch_bounds__(256) resid_kernel(const int* __restrict__ pop,
             many &= many - 1;
             const int vb = __shfl_sync(0xffffffffu, v, src), bb = __shfl_sync(0xffffffffu, b, src),
                       eb = __shfl_sync(0xffffffffu, e, src);
-            for (int p = bb + lane; p < eb; p += 32) resid_pair(bm, T, col, vb, __ldg(col + p), c0, c1, c2);
+            for (int p = bb + lane; p < eb; p += 32) arc(vb, __ldg(col + p));
         }
+    }
+    if (kOnce) {
+        // a row with repeated genes counts a node once per gene equal to its first deleted neighbour
+        auto times = [&](int v) {
+            if (!repeated) return 1;
+            int c = 0;
+            for (int j = 0; j < k; ++j) c += genes[j] == v;
+            return c;
+        };
+        bool more;
+        do {  // again while the list overflows (listed nodes leave the bitmap)
+            __syncthreads();
+            if (t == 0) s_count = 0;
+            __syncthreads();
+            for (int w0 = warp * 32; w0 < words; w0 += nwarps * 32) {
+                const int w = w0 + lane;
+                const unsigned bits = w < words ? twice[w] & ~bm[w] : 0u;
+                if (!__any_sync(0xffffffffu, bits)) continue;
+                const int cnt = __popc(bits);
+                int incl = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                int first = 0;
+                if (lane == 31) first = atomicAdd(&s_count, incl);
+                int at = __shfl_sync(0xffffffffu, first, 31) + incl - cnt;
+                unsigned left = bits;
+                for (; left && at < kResidList; left &= left - 1, ++at) s_list[at] = 32 * w + __ffs(left) - 1;
+                if (w < words) twice[w] = left;
+            }
+            __syncthreads();
+            const int listed = min(s_count, kResidList);
+            more = s_count > kResidList;
+            for (int i = t; i < listed; i += blockDim.x)
+                resid_node(bm, T, row_ptr, col, -1, s_list[i], c0, c1, c2, times);
+        } while (more);
     }
     for (int o = 16; o > 0; o >>= 1) {
         c0 += __shfl_down_sync(0xffffffffu, c0, o);
@@ -328,47 +445,27 @@ __global__ void __launch_bounds__(256) resid_kernel(const int* __restrict__ pop,
             z += red[2][w];
         }
         out[r].c = make_int4(x, y, z, 0);
-    }
-}
-
-// Mean and standard deviation of each of the three counts over `rows` residual records (one CTA:
-// exact int64 sums, then FP64 in a fixed order with explicit rounding: mean = S1 / rows,
-// var = S2 / rows - mean^2, sd = max(sqrt(var), 1)); ms[0..2] = means, ms[3..5] = deviations.
-__global__ void __launch_bounds__(256) resid_stats_kernel(const ResidRow* __restrict__ r, int rows,
-                                                          double* __restrict__ ms) {
-    __shared__ long long s1[3][256], s2[3][256];
-    long long a[3] = {0, 0, 0}, b[3] = {0, 0, 0};
-    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-        const int4 c = r[i].c;
-        const long long v[3] = {c.x, c.y, c.z};
+        const unsigned long long c[3] = {(unsigned long long)x, (unsigned long long)y, (unsigned long long)z};
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            a[j] += v[j];
-            b[j] += v[j] * v[j];
+            atomicAdd(&sums[j], c[j]);
+            atomicAdd(&sums[3 + j], c[j] * c[j]);
         }
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        s1[j][threadIdx.x] = a[j];
-        s2[j][threadIdx.x] = b[j];
+        __threadfence();
+        s_last = atomicAdd(&sums[6], 1ull) == (unsigned long long)rows - 1;
     }
     __syncthreads();
-    for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                s1[j][threadIdx.x] += s1[j][threadIdx.x + w];
-                s2[j][threadIdx.x] += s2[j][threadIdx.x + w];
-            }
-        __syncthreads();
+    if (!s_last || t >= 7) return;
+    __threadfence();
+    if (t < 3) {
+        const double s1 = (double)(long long)__ldcg(&sums[t]), s2 = (double)(long long)__ldcg(&sums[3 + t]);
+        const double mean = __ddiv_rn(s1, (double)rows);
+        const double var = __dsub_rn(__ddiv_rn(s2, (double)rows), __dmul_rn(mean, mean));
+        ms[t] = mean;
+        ms[3 + t] = fmax(__dsqrt_rn(fmax(var, 0.0)), 1.0);
     }
-    if (threadIdx.x < 3) {
-        const int j = threadIdx.x;
-        const double mean = __ddiv_rn((double)s1[j][0], (double)rows);
-        const double var = __dsub_rn(__ddiv_rn((double)s2[j][0], (double)rows), __dmul_rn(mean, mean));
-        ms[j] = mean;
-        ms[3 + j] = fmax(__dsqrt_rn(fmax(var, 0.0)), 1.0);
-    }
+    __syncwarp(0x7Fu);
+    sums[t] = 0ull;
 }
 
 // z of every record from the statistics: z = float((c - mean) / sd), the FP64 operations
@@ -980,16 +1077,19 @@ struct gapa_surrogate {
          *dZ1 = nullptr, *dZ1T = nullptr;
     float *y = nullptr, *dy = nullptr, *dX = nullptr, *loss = nullptr, *tbuf = nullptr;
     ResidRow* resid = nullptr;   // residual-degree counts (and their z) of the rows of the last forward
-    int4* nbr = nullptr;         // per node: first arc, degree, its two lowest-degree neighbours
+    int4* nbr = nullptr;         // per node: its four lowest-degree neighbours
     const int* row_ptr = nullptr;  // the context's CSR (original node ids)
     const int* col = nullptr;
-    size_t resid_smem = 0;       // deletion bitmap bytes of resid_kernel
+    size_t resid_smem = 0;       // bytes of one bitmap of resid_kernel
+    bool resid_once = false;     // its three bitmaps fit in shared memory
+    unsigned* low = nullptr;     // bitmap of the nodes of degree one and two
     int* batch_rows = nullptr;
     double* stats = nullptr;
     int tau = 0;
     // embedding gradient: occurrences per node, list offsets (n + 1), fill cursors, block totals,
     // and the rows of every node's list
     int *emb_cnt = nullptr, *emb_off = nullptr, *emb_cur = nullptr, *emb_blk = nullptr, *rows_of = nullptr;
+    unsigned long long* rsums = nullptr;  // running sums of resid_kernel (7, zero between launches)
     double* rstats = nullptr;  // means and deviations of the residual counts of the last rows computed
     long long* emb_q = nullptr;  // the rounded gradient terms [rows][64] of the last training step
     int emb_q_rows = 0;
@@ -1032,9 +1132,15 @@ int round16(int x) { return (x + 15) & ~15; }
 // Residual-degree counts of `rows` deletion sets into s->resid, standardised over those rows.
 int compute_resid(gapa_surrogate* s, const int32_t* pop, int rows, int k, cudaStream_t st) {
     if (rows <= 0) return GAPA_OK;
-    ProfileScope prof(s->ctx, st, 2, 3);
-    resid_kernel<<<rows, 256, s->resid_smem, st>>>(pop, rows, k, s->n, s->nbr, s->col, s->resid);
-    resid_stats_kernel<<<1, 256, 0, st>>>(s->resid, rows, s->rstats);
+    ProfileScope prof(s->ctx, st, 2, 2);
+    // 256 threads per row where that fills the device's 2048 per SM, more where rows are few or their
+    // bitmaps keep CTAs off an SM (256 rows of 1500 genes, n = 30011: 102 us by the former per-arc kernel at 256 threads, 30 us at 1024)
+    const size_t smem = s->resid_once ? 3 * s->resid_smem : s->resid_smem;
+    const size_t per_sm = s->ctx->smem_per_sm / (smem + (s->resid_once ? 14336 : 10240));
+    int T = 256;
+    while (T < 1024 && (per_sm * T < 2048 || (long long)rows * T < 2048ll * s->ctx->num_sms)) T *= 2;
+    const auto kern = s->resid_once ? resid_kernel<true> : resid_kernel<false>;
+    kern<<<rows, T, smem, st>>>(pop, rows, k, s->n, s->low, s->nbr, s->row_ptr, s->col, s->resid, s->rsums, s->rstats);
     resid_z_kernel<<<(rows + 127) / 128, 128, 0, st>>>(s->resid, rows, s->rstats);
     GAPA_CUDA(cudaGetLastError());
     return GAPA_OK;
@@ -1215,7 +1321,7 @@ void free_surrogate(gapa_surrogate* s) {
     void* ps[] = {s->P, s->M, s->V, s->G, s->Gi, s->W1b, s->W1tb, s->W2b, s->W2tb, s->Eb, s->logdeg, s->deg,
                   s->X, s->XT, s->H1, s->H1T, s->H2, s->dZ2, s->dZ2T, s->dZ1, s->dZ1T, s->y, s->dy, s->dX,
                   s->loss, s->tbuf, s->batch_rows, s->stats, s->resid, s->nbr, s->emb_cnt, s->emb_off,
-                  s->emb_cur, s->emb_blk, s->rows_of, s->rstats, s->emb_q};
+                  s->emb_cur, s->emb_blk, s->rows_of, s->rstats, s->rsums, s->low, s->emb_q};
     for (void* p : ps) cudaFree(p);
 }
 
@@ -1246,12 +1352,17 @@ int gapa_surrogate_create(gapa_surrogate** out, gapa_ctx* ctx, const gapa_surrog
         delete s;
         return gapa_fail(GAPA_ERR_INVALID_ARG, "n = %d: the deletion bitmap does not fit in shared memory", ctx->g.n);
     }
-    if (s->resid_smem > 48 * 1024 &&
-        cudaFuncSetAttribute(resid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->resid_smem) !=
-            cudaSuccess) {
+    size_t once_max = 0, plain_max = 0;
+    if (gapa_set_smem_limit((const void*)resid_kernel<true>, ctx->smem_optin, &once_max) != GAPA_OK ||
+        gapa_set_smem_limit((const void*)resid_kernel<false>, ctx->smem_optin, &plain_max) != GAPA_OK) {
         cudaGetLastError();
         delete s;
         return gapa_fail(GAPA_ERR_CUDA, "shared memory limit of the residual-degree kernel");
+    }
+    s->resid_once = 3 * s->resid_smem <= once_max;
+    if (s->resid_smem > plain_max) {
+        delete s;
+        return gapa_fail(GAPA_ERR_INVALID_ARG, "n = %d: the deletion bitmap does not fit in shared memory", ctx->g.n);
     }
     s->L = make_layout(s->n);
     auto bail = [&](int rc) {
@@ -1268,7 +1379,9 @@ int gapa_surrogate_create(gapa_surrogate** out, gapa_ctx* ctx, const gapa_surrog
         cudaMalloc(&s->deg, (size_t)s->n * 4) || cudaMalloc(&s->loss, 4) || cudaMalloc(&s->stats, 16) ||
         cudaMalloc(&s->nbr, (size_t)s->n * sizeof(int4)) || cudaMalloc(&s->emb_cnt, (size_t)s->n * 4) ||
         cudaMalloc(&s->emb_off, ((size_t)s->n + 1) * 4) || cudaMalloc(&s->emb_cur, (size_t)s->n * 4) ||
-        cudaMalloc(&s->emb_blk, ((size_t)(s->n + 1023) / 1024 + 1) * 4) || cudaMalloc(&s->rstats, 6 * sizeof(double))) {
+        cudaMalloc(&s->emb_blk, ((size_t)(s->n + 1023) / 1024 + 1) * 4) || cudaMalloc(&s->rstats, 6 * sizeof(double)) ||
+        cudaMalloc(&s->rsums, 7 * sizeof(unsigned long long)) ||
+        cudaMalloc(&s->low, s->resid_smem)) {
         cudaGetLastError();
         return bail(gapa_fail(GAPA_ERR_OOM, "surrogate parameters"));
     }
@@ -1286,6 +1399,8 @@ int gapa_surrogate_create(gapa_surrogate** out, gapa_ctx* ctx, const gapa_surrog
     cudaMemcpy(s->deg, dg.data(), dg.size() * 4, cudaMemcpyHostToDevice);
     cudaStream_t st = ctx->stream;
     nbr_table_kernel<<<ctx->num_sms * 4, 256, 0, st>>>(s->row_ptr, s->col, s->n, s->nbr);
+    low_degree_kernel<<<ctx->num_sms, 128, 0, st>>>(s->row_ptr, s->n, s->low);
+    cudaMemsetAsync(s->rsums, 0, 7 * sizeof(unsigned long long), st);
     cudaMemsetAsync(s->P, 0, np * 4, st);
     cudaMemsetAsync(s->M, 0, np * 4, st);
     cudaMemsetAsync(s->V, 0, np * 4, st);
