@@ -192,10 +192,9 @@ int gapa_batch_get_teams(gapa_batch* batch, int32_t* teams /* [num] */);
  * 16384, 32768, 65536) time each feasible team count on the initial
  * population and keep the fastest; choices are cached per device name in
  * the JSON file `cache_path` (NULL: no cache).  Batched instances follow
- * their context's fitness kernel setting as single runs do: AUTO takes the
- * cut-local kernel above 2048 nodes (in each team's slice, with the
- * operator kernels' cost estimates), TREE_LOCAL always, anything else the
- * full TREE pipeline. */
+ * their context's fitness kernel setting as single runs do: AUTO and
+ * TREE_LOCAL take the cut-local kernel (in each team's slice), anything else
+ * the full TREE pipeline. */
 int gapa_batch_autotune(gapa_batch* batch, const char* cache_path);
 
 /* Run every instance for `gens` generations from its initialisation.
@@ -291,19 +290,19 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * first live node scan their adjacency (when their adjacency is shorter than
  * the list of non-tree edges) or unites along every non-tree edge.
  * TREE_JOIN and TREE_SCAN force one of the two (for tests and measurement).
- * TREE_LOCAL reaches the same pieces with work local to the deletion: the
- * tree parents are bulk-copied into the labels, only the children of deleted
- * nodes are re-picked, and only the pieces whose root is not the first live
- * node are listed (level by level down the tree) and scanned; a member whose
- * list outgrows the kernel's shared memory, or with repeated genes, takes
- * the TREE path.  It needs n <= 65536 and a BFS tree whose children carry
- * consecutive numbers (always so for the upload's numbering).
+ * TREE_LOCAL reaches the same components with work local to the deletion: the
+ * tree parents are bulk-copied into the labels, the children of deleted nodes
+ * take a live lower-numbered neighbour (or are united with higher-numbered
+ * ones), and only the classes left apart from the first live node's are listed
+ * and searched; a member with repeated genes, or whose lists outgrow the
+ * kernel's shared memory, takes the TREE path.  It needs a graph whose 16-bit
+ * ids and labels fit in shared memory (n up to about 56,000 on GB300).
  * SAMPLED joins every live node to its first two live neighbours, takes the
  * tree of the highest-degree live node as the giant tree and lets only nodes
  * outside it scan their whole adjacency; EDGES runs union-find over every
- * undirected edge.  AUTO (the default) is TREE_LOCAL where it applies and
- * the graph has more than 2048 nodes, else TREE.  Where the labels do not fit
- * in shared memory (n above about 56,000 on GB300), AUTO runs SPARSE
+ * undirected edge.  AUTO (the default) is TREE_LOCAL where it applies and the
+ * mean degree is at least 3 (5 up to 2048 nodes), else TREE.  Where the labels
+ * do not fit in shared memory (n above about 56,000 on GB300), AUTO runs SPARSE
  * (below), the TREE settings run the same phases on labels in global memory,
  * eight members interleaved per 32-byte sector, and EDGES and SAMPLED run one
  * CTA per member over a global label array. */

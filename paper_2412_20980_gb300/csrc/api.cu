@@ -46,6 +46,8 @@ void free_graph(DeviceGraph& g) {
     cudaFree(g.crep);
     cudaFree(g.nroot);
     cudaFree(g.csize);
+    void* cut_ptrs[] = {g.lc.par, g.lc.gene, g.lc.lower, g.lc.higher, g.lc.near, g.lc.roots, g.lc.cost};
+    for (void* q : cut_ptrs) cudaFree(q);
     DeviceForest& a = g.alt;
     void* alt_ptrs[] = {a.perm, a.tparent, a.palt, a.lo_ptr, a.lo_col, a.kids, a.roots, a.cut, a.fptr, a.fcol16,
                         a.nontree, a.sz, a.pre, a.at, a.crep, a.nroot, a.csize};
@@ -346,9 +348,8 @@ std::vector<int32_t> hub_last_perm(int32_t n, const std::vector<int32_t>& rp, co
 
 // Device copy of a forest (nullptr members on failure, which the caller frees).
 int upload_forest(const ForestHost& f, int32_t n, DeviceForest& d) {
-    const size_t par_ints = gapa_dev::tree16l_lab_ints(n);
-    std::vector<int32_t> par(f.tparent);
-    par.resize(par_ints, 0);
+    const std::vector<int32_t>& par = f.tparent;
+    const size_t par_ints = (size_t)n;
     std::vector<uint16_t> f16(f.fcol.begin(), f.fcol.end());
     auto up = [](void** dst, const void* src, size_t bytes) {
         if (cudaMalloc(dst, std::max<size_t>(bytes, 16)) != cudaSuccess) return false;
@@ -375,6 +376,61 @@ int upload_forest(const ForestHost& f, int32_t n, DeviceForest& d) {
         cudaGetLastError();
         return gapa_fail(GAPA_ERR_OOM, "second forest of %d nodes", n);
     }
+    return GAPA_OK;
+}
+
+// Tables of the cut-local kernel (see CutTables) from the BFS forest, the graph (rows by original id)
+// and the children ranges by number.
+int upload_cut_tables(const BfsForest& bf, const std::vector<int32_t>& rp, const std::vector<int32_t>& col, int32_t n,
+                      const std::vector<int4>& kids, CutTables& t) {
+    const uint32_t none = 0xFFFFu;
+    std::vector<int32_t> inv((size_t)n), roots, cost((size_t)n);
+    for (int32_t v = 0; v < n; ++v) inv[bf.perm[v]] = v;
+    auto degree = [&](int32_t b) { return rp[inv[b] + 1] - rp[inv[b]]; };
+    std::vector<uint16_t> par(gapa_dev::tree16_lab_bytes(n) / 2, 0);
+    std::vector<uint2> gene((size_t)n);
+    std::vector<uint2> low((size_t)n), high((size_t)n);
+    std::vector<uint16_t> near((size_t)n * 8, 0xFFFFu);
+    t.singles = 0;
+    for (int32_t b = 0; b < n; ++b) {
+        const int32_t v = inv[b];
+        const bool single = degree(b) == 0;
+        par[b] = (uint16_t)bf.tparent[b];
+        gene[v] = make_uint2((uint32_t)b | (uint32_t)(kids[b].x & 0xFFFF) << 16,
+                             (uint32_t)kids[b].y | (single ? 1u << 16 : 0u));
+        cost[v] = kids[b].y + 1;
+        t.singles += single;
+        if (bf.tparent[b] == b && !single) roots.push_back(b);
+        // lower-numbered neighbours after the parent: the first three and the last
+        uint32_t lower[4] = {none, none, none, none}, higher[4] = {none, none, none, none};
+        const int32_t l0 = bf.lo_ptr[b] + 1, l1 = bf.lo_ptr[b + 1];
+        for (int32_t i = 0; i < 3 && l0 + i < l1; ++i) lower[i] = (uint32_t)bf.lo_col[l0 + i];
+        if (l1 - l0 > 3) lower[3] = (uint32_t)bf.lo_col[l1 - 1];
+        for (int32_t i = 0; i < 8 && rp[v] + i < rp[v + 1]; ++i)
+            near[(size_t)b * 8 + i] = (uint16_t)bf.perm[col[rp[v] + i]];
+        // the four of highest degree among the higher-numbered ones outside its subtree's first level
+        for (int32_t e = rp[v]; e < rp[v + 1]; ++e) {
+            const int32_t w = bf.perm[col[e]];
+            if (w < b || bf.tparent[w] == b) continue;
+            uint32_t x = (uint32_t)w;
+            for (int i = 0; i < 4 && x != none; ++i)
+                if (higher[i] == none || degree((int32_t)x) > degree((int32_t)higher[i])) std::swap(x, higher[i]);
+        }
+        low[b] = make_uint2(lower[0] | lower[1] << 16, lower[2] | lower[3] << 16);
+        high[b] = make_uint2(higher[0] | higher[1] << 16, higher[2] | higher[3] << 16);
+    }
+    auto up = [](void** dst, const void* src, size_t bytes) {
+        return cudaMalloc(dst, std::max<size_t>(bytes, 16)) == cudaSuccess &&
+               (bytes == 0 || cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess);
+    };
+    if (!(up((void**)&t.par, par.data(), 2 * par.size()) && up((void**)&t.gene, gene.data(), sizeof(uint2) * (size_t)n) &&
+          up((void**)&t.lower, low.data(), sizeof(uint2) * (size_t)n) &&
+          up((void**)&t.higher, high.data(), sizeof(uint2) * (size_t)n) && up((void**)&t.near, near.data(), 2 * near.size()) &&
+          up((void**)&t.roots, roots.data(), 4 * roots.size()) && up((void**)&t.cost, cost.data(), 4 * (size_t)n))) {
+        cudaGetLastError();
+        return gapa_fail(GAPA_ERR_OOM, "cut-local tables of %d nodes", n);
+    }
+    t.num_roots = (int)roots.size();
     return GAPA_OK;
 }
 
@@ -500,8 +556,7 @@ int enqueue_generation(gapa_ctx* c, const GaParams& p0, int lambda, const int32_
     const int evaluated = (p.flags & GAPA_FLAG_MU_PLUS_LAMBDA) ? lambda : p.s;
     unsigned* est = gapa_fitness_uses_estimates(c, evaluated) ? gapa_estimate_buffer(c) : nullptr;
     if (est) {
-        p.est_cut = c->g.cut;
-        if (c->g.has_alt) p.est_cut2 = c->g.alt.cut;
+        gapa_estimate_tables(c, &p.est_cut, &p.est_cut2);
         p.est_out = est;
         p.est_stride = kOrderCap;
     }
@@ -909,11 +964,11 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     g.num_nontree = (int)bf.nontree.size();
     g.mean_deg_x16 = n > 0 ? (int)((16 * nnz + n - 1) / n) : 0;
     // 16-bit ids only on the shared-memory path (labels + deleted-node bitmap)
-    g.packed16 = n <= 65536 && gapa_dev::tree16_smem_bytes(n) <= c->fit_smem_max;
+    // (the limit: 4 bytes per node and a bitmap within shared memory, n <= about 57,000)
+    g.packed16 = n < gapa_dev::kDead16 && gapa_dev::tree32_smem_bytes(n) <= c->fit_smem_max;
     const size_t nt_bytes = (g.packed16 ? 4 : 8) * std::max<size_t>(bf.nontree.size(), 4);
-    const size_t par_ints = gapa_dev::tree16l_lab_ints(n);  // padded for the bulk copy of the cut-local kernel
     if (cudaMalloc(&g.perm, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
-        cudaMalloc(&g.tparent, sizeof(int32_t) * par_ints) != cudaSuccess ||
+        cudaMalloc(&g.tparent, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
         cudaMalloc(&g.lo_ptr, sizeof(int32_t) * ((size_t)n + 1)) != cudaSuccess ||
         cudaMalloc(&g.lo_col, sizeof(int32_t) * std::max<size_t>(bf.lo_col.size(), 1)) != cudaSuccess ||
         cudaMalloc(&g.nontree, nt_bytes) != cudaSuccess) {
@@ -922,14 +977,10 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
         return gapa_fail(GAPA_ERR_OOM, "BFS forest of %d nodes", n);
     }
     GAPA_CUDA(cudaMemcpy(g.perm, bf.perm.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
-    {
-        std::vector<int32_t> par(bf.tparent);
-        par.resize(par_ints, 0);
-        GAPA_CUDA(cudaMemcpy(g.tparent, par.data(), sizeof(int32_t) * par_ints, cudaMemcpyHostToDevice));
-    }
+    GAPA_CUDA(cudaMemcpy(g.tparent, bf.tparent.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
     if (g.packed16) {
-        // cut-local TREE kernel: children ranges (consecutive in BFS order), component roots, and a
-        // list region as large as two members per SM allow (one per SM when the labels need it)
+        // cut-local TREE kernel and forest-piece kernel: children ranges (consecutive in BFS order) and
+        // component roots
         std::vector<int4> kids((size_t)n);
         bool contiguous = true;
         for (int32_t b = 0; b < n; ++b) kids[b] = make_int4(b, 0, 0, 0);
@@ -940,19 +991,12 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
             else if (kids[p].x + kids[p].y != x) contiguous = false;
             kids[p].y += 1;
         }
-        const int team = gapa_fitness_block_for(n);
-        const size_t fixed = par_ints * 4 + 48, min_list = gapa_dev::tree16l_min_list_bytes(n, team);
-        const size_t want = std::max(min_list, ((((size_t)n * 2) + 15) & ~(size_t)15) + gapa_dev::tree16l_bitmap_bytes(n) +
-                                                   gapa_dev::tree16l_scratch_bytes(team));
-        // two members per SM: half the SM's shared memory, less the runtime's reserve and the
-        // kernel's static shared memory (under 1 KB)
-        const size_t per_block = c->smem_per_sm / 2, other = c->smem_reserved + 1024;
-        const size_t two_per_sm = per_block > other ? per_block - other : 0;
-        size_t budget = fixed + min_list <= two_per_sm ? two_per_sm : c->fit_smem_max;
-        budget = std::min(budget, c->fit_smem_max);
-        size_t list_bytes = 0;
-        if (contiguous && fixed + min_list <= budget) list_bytes = std::min(want, (budget - fixed) & ~(size_t)15);
-        if (list_bytes) {
+        if (contiguous && gapa_dev::tree16l_smem_bytes(n, gapa_dev::tree16l_min_list_bytes(n, g.mean_deg_x16)) <= c->fit_smem_max) {
+            const int lrc = upload_cut_tables(bf, rp, sorted, n, kids, g.lc);
+            if (lrc != GAPA_OK) {
+                free_graph(g);
+                return lrc;
+            }
             // cost estimate of deleting node b: the nodes below those children of b whose only lower
             // neighbour is b (they become roots of pieces to be listed)
             std::vector<int32_t> below((size_t)n, 1), cut((size_t)n, 0);
@@ -976,7 +1020,6 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
                 GAPA_CUDA(cudaMemcpy(g.roots, bf.roots.data(), sizeof(int32_t) * bf.roots.size(),
                                      cudaMemcpyHostToDevice));
             g.num_roots = (int)bf.roots.size();
-            g.local_list_bytes = (int)list_bytes;
             {
                 // subtree intervals of the forest-piece kernel
                 const ForestIntervals fi = forest_intervals(bf.tparent, bf.lo_ptr, bf.lo_col);
@@ -995,8 +1038,7 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
                 }
                 g.tree_pc = fi.tree_pc;
             }
-            // the second forest, numbered with the top hubs last (about 0.5 % of the nodes, 8 to 256):
-            // members that delete hubs cut it far less
+            // the second forest, numbered with the top hubs last (about 0.5 % of the nodes, 8 to 256)
             const int hubs = std::max(8, std::min(256, n / 200));
             if (n > 4 * hubs) {
                 const ForestHost fb = forest_host(n, rp, sorted, hub_last_perm(n, rp, sorted, hubs));

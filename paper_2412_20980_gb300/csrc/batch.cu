@@ -30,7 +30,6 @@ struct gapa_batch {
     int* status = nullptr;          // ctxs[0]'s status word
     std::vector<int> teams;         // members per CTA per instance
     std::vector<int> use_local;     // per instance: the cut-local kernel
-    unsigned* d_est = nullptr;      // cost estimates of the local instances' rows (two per row)
     // device memory
     BatchDesc* d_desc = nullptr;
     int2* d_rows = nullptr;
@@ -52,11 +51,13 @@ struct gapa_batch {
 
 namespace {
 
-size_t need16(int n) { return gapa_dev::tree16_smem_bytes(n); }
+// Slice of the full pipeline (team counts are bounded by it).
+size_t need16(int n) { return gapa_dev::tree32_smem_bytes(n); }
 
-// Slice of one team of T threads that also holds the cut-local kernel's layout (minimum list region).
-size_t need_local(int n, int T) {
-    return gapa_dev::tree16l_lab_ints(n) * 4 + gapa_dev::tree16l_min_list_bytes(n, T) + 48;
+// Slice of one team that also holds the cut-local kernel's layout with a list of n / 4 entries.
+size_t need_local(int n, int mean_deg_x16) {
+    return gapa_dev::tree16l_smem_bytes(n, std::max(gapa_dev::tree16l_min_list_bytes(n, mean_deg_x16),
+                                                    gapa_dev::tree16l_bitmap_bytes(n) + (((size_t)n / 2 + 15) & ~(size_t)15)));
 }
 
 // Slice bytes of instance x at c teams: the cut-local layout where the graph has it and c slices of
@@ -76,8 +77,6 @@ int default_teams(int n, size_t max_dyn) {
 }
 
 void free_batch_device(gapa_batch* b) {
-    cudaFree(b->d_est);
-    b->d_est = nullptr;
     cudaFree(b->d_desc);
     cudaFree(b->d_rows);
     cudaFree(b->d_pk);
@@ -97,8 +96,8 @@ void free_batch_device(gapa_batch* b) {
 size_t slice_need(const gapa_batch* b, int x, int c) {
     const DeviceGraph& g = b->ctxs[x]->g;
     const size_t full = need16(g.n);
-    if (!b->desc[x].kids || !b->use_local[x]) return full;  // the instance runs the full pipeline
-    const size_t local = std::max(full, need_local(g.n, 1024 / c));
+    if (!b->use_local[x]) return full;  // the instance runs the full pipeline
+    const size_t local = need_local(g.n, g.mean_deg_x16);
     return (size_t)c * ((local + 15) & ~(size_t)15) <= b->fit_max_dyn ? local : full;
 }
 
@@ -140,11 +139,11 @@ int build_packets(gapa_batch* b) {
         BatchDesc& d = b->desc[i];
         d.teams = b->teams[i];
         // the cut-local kernel where the instance's slice holds its layout
-        const int n = b->ctxs[i]->g.n, T = 1024 / d.teams;
+        const int n = b->ctxs[i]->g.n;
         const size_t slice = (b->fit_smem / (size_t)d.teams) & ~(size_t)15;
-        const size_t fixed = gapa_dev::tree16l_lab_ints(n) * 4 + 48;
+        const size_t fixed = gapa_dev::tree16l_smem_bytes(n, 0);
         d.list_bytes = 0;
-        if (d.kids && b->use_local[i] && slice >= fixed + gapa_dev::tree16l_min_list_bytes(n, T))
+        if (b->use_local[i] && slice >= fixed + gapa_dev::tree16l_min_list_bytes(n, d.mean_deg_x16))
             d.list_bytes = (int)((slice - fixed) & ~(size_t)15);
     }
     return GAPA_OK;
@@ -346,41 +345,13 @@ int gapa_batch_create(gapa_batch** out, int32_t num, gapa_ctx* const* ctxs, cons
         d.fcol16 = dg.fcol16;
         d.mean_deg_x16 = dg.mean_deg_x16;
         d.objective = b->ctxs[i]->objective;
-        const int variant = b->ctxs[i]->fitness_variant;
-        if (dg.local_list_bytes > 0 && (variant == GAPA_FITNESS_TREE_LOCAL ||
-                                        (variant == GAPA_FITNESS_AUTO && dg.n > 2048))) {
-            // the cut-local kernel as on a single context: the operator kernels write every row's
-            // estimates under both forests, members estimated to shatter both run the full pipeline
+        // the cut-local kernel as on a single context
+        if (gapa_fitness_local(b->ctxs[i])) {
             b->use_local[i] = 1;
-            d.alt = dg.alt;
-            d.tparent = dg.tparent;
-            d.kids = dg.kids;
-            d.roots = dg.roots;
-            d.num_roots = dg.num_roots;
+            d.lc = dg.lc;
         }
         b->teams[i] = default_teams(dg.n, b->fit_max_dyn);
         for (int r = 0; r < g.pop; ++r) rows.push_back(make_int2(i, r));
-    }
-    // cost estimates of the cut-local instances' rows: two per row (first forest, second forest)
-    size_t est_total = 0;
-    for (int i = 0; i < num; ++i)
-        if (b->use_local[i]) est_total += 2 * (size_t)cfgs[i].pop;
-    if (est_total) {
-        if (cudaMalloc(&b->d_est, sizeof(unsigned) * est_total) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(gapa_fail(GAPA_ERR_OOM, "batch cost estimates"));
-        }
-        size_t eo = 0;
-        for (int i = 0; i < num; ++i) {
-            if (!b->use_local[i]) continue;
-            BatchDesc& d = b->desc[i];
-            const DeviceGraph& dg = ctxs[i]->g;
-            d.p.est_cut = dg.cut;
-            d.p.est_cut2 = dg.has_alt ? dg.alt.cut : nullptr;
-            d.p.est_out = b->d_est + eo;
-            d.p.est_stride = cfgs[i].pop;
-            eo += 2 * (size_t)cfgs[i].pop;
-        }
     }
     if (cudaMemcpy(b->d_rows, rows.data(), sizeof(int2) * rows.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(gapa_fail(GAPA_ERR_CUDA, "uploading the row table"));

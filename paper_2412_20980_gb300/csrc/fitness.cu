@@ -287,49 +287,33 @@ struct GraphArgs {
     int join_mode;
     int mean_deg_x16;
     int objective;
-    const int4* kids;
-    const int* roots;
-    int num_roots;
+    CutTables lc;    // cut-local kernel
     int list_bytes;
-    const unsigned* est;  // cut-local kernel: per-member cost estimates (may be null)
-    DeviceForest alt;     // cut-local kernel: the second forest (alt.perm null: none)
 };
 
 enum Variant : int { V_EDGES = 0, V_SAMPLED = 1, V_TREE16 = 2, V_TREE32 = 3, V_TREE16L = 4 };
 
+__device__ __forceinline__ gapa_dev::Tree16Graph tree16_graph(const GraphArgs& g) {
+    return gapa_dev::Tree16Graph{g.n,    g.perm,   g.palt,      g.lo_ptr,       g.lo_col,    (const unsigned*)g.nontree,
+                                 g.num_nontree, g.fptr, g.fcol16, g.join_mode, g.mean_deg_x16, g.objective,
+                                 g.lc,   g.list_bytes, gapa_dev::tree16l_tops_max(g.n, g.mean_deg_x16)};
+}
+
 template <int kVar>
-__device__ __forceinline__ void member_pc(volatile int* lab, const GraphArgs& g, const int* __restrict__ genes, int k, int m,
-                                          long long* out, int* status, long long* red, int* sh_root,
-                                          bool use_alt = false) {
+__device__ __forceinline__ void member_pc(volatile int* lab, const GraphArgs& g, const int* __restrict__ genes, int k,
+                                          long long* out, int* status, long long* red, int* sh_root) {
     if (kVar == V_TREE16 || kVar == V_TREE16L) {
-        // the whole CTA is one team; the deleted-node bitmap sits right after the labels
+        // the whole CTA is one team; the deleted-node bitmap (cut-local: the list region) sits right after
+        // the labels
         const gapa_dev::Team tm{(int)threadIdx.x, (int)blockDim.x, 0};
-        // the cut-local kernel leaves members expected to list over a quarter of the nodes (the
-        // BFS tree shattered) to the full pipeline from the start
-        const bool full = kVar == V_TREE16 || (g.est && __ldg(&g.est[m]) > (unsigned)(g.n / 4));
-        unsigned* region = (unsigned*)(lab + gapa_dev::tree16l_lab_ints(g.n));
-        int* scal = (int*)region + g.list_bytes / 4;
-        if (kVar == V_TREE16L && use_alt && !full) {
-            // the second forest: the same graph in its own numbering (its own constant record, so
-            // that every field stays a kernel-parameter read)
-            const DeviceForest& a = g.alt;
-            const gapa_dev::Tree16Graph tb{g.n,           a.perm,          a.palt,          a.lo_ptr,
-                                           a.lo_col,      a.nontree,       a.num_nontree,   a.fptr,
-                                           a.fcol16,      g.join_mode,     g.mean_deg_x16,  g.objective,
-                                           a.tparent,     a.kids,          a.roots,         a.num_roots,
-                                           g.list_bytes};
-            gapa_dev::tree16_member_local(tm, lab, region, scal, tb, genes, k, out, red, status);
-            return;
+        const gapa_dev::Tree16Graph t16 = tree16_graph(g);
+        if (kVar == V_TREE16) {
+            gapa_dev::tree32_member(tm, lab, (unsigned*)(lab + g.n), t16, genes, k, out, red, status);
+        } else {
+            unsigned* region = (unsigned*)(lab + gapa_dev::tree16_lab_bytes(g.n) / 4);
+            gapa_dev::tree16_member_local(tm, reinterpret_cast<volatile gapa_dev::lab_t*>(lab), region,
+                                          (int*)region + g.list_bytes / 4, t16, genes, k, out, red, status);
         }
-        const gapa_dev::Tree16Graph t16{g.n,           g.perm,          g.palt,          g.lo_ptr,
-                                        g.lo_col,      (const unsigned*)g.nontree,      g.num_nontree,
-                                        g.fptr,        g.fcol16,        g.join_mode,     g.mean_deg_x16,
-                                        g.objective,   g.tparent,       g.kids,          g.roots,
-                                        g.num_roots,   g.list_bytes};
-        if (full)
-            gapa_dev::tree16_member(tm, lab, (unsigned*)(lab + g.n), t16, genes, k, out, red, status);
-        else
-            gapa_dev::tree16_member_local(tm, lab, region, scal, t16, genes, k, out, red, status);
         return;
     }
     if (kVar == V_TREE32) {
@@ -390,9 +374,19 @@ __global__ void __launch_bounds__(1024) cc_smem_kernel(GraphArgs g, const int* _
     extern __shared__ int smem_lab[];
     __shared__ long long red[32];
     __shared__ int sh_root;
-    const int e = order ? __ldg(&order[blockIdx.x]) : (int)blockIdx.x;
-    const int i = e & 0x3FFFFFFF;  // bit 30: evaluate on the second forest
-    member_pc<kVar>(smem_lab, g, pop + (size_t)i * k, k, i, &fit[i], status, red, &sh_root, (e >> 30) & 1);
+    const int i = order ? __ldg(&order[blockIdx.x]) : (int)blockIdx.x;
+    member_pc<kVar>(smem_lab, g, pop + (size_t)i * k, k, &fit[i], status, red, &sh_root);
+}
+
+// The cut-local kernel, at most 32 registers per thread: 2048 threads per SM.
+__global__ void __launch_bounds__(1024, 2) cc_local_kernel(const __grid_constant__ GraphArgs g,
+                                                           const int* __restrict__ pop, int k,
+                                                           long long* __restrict__ fit, int* status,
+                                                           const int* __restrict__ order) {
+    extern __shared__ __align__(16) int smem_loc[];
+    __shared__ long long red[32];
+    const int i = order ? __ldg(&order[blockIdx.x]) : (int)blockIdx.x;
+    member_pc<V_TREE16L>(smem_loc, g, pop + (size_t)i * k, k, &fit[i], status, red, nullptr);
 }
 
 // Cost estimate of every member for the cut-local kernel under each forest:
@@ -443,35 +437,34 @@ __global__ void __launch_bounds__(128) local_cost_kernel(const int* __restrict__
     }
 }
 
-// Members by decreasing bit length of their lower estimate (a counting sort
-// over the 33 values of its count of leading zeros, in one CTA; the order
-// within a class is arbitrary).  order[i] = member | 1 << 30 when the second
-// forest has the lower estimate; est_min[m] = the lower estimate.
-__global__ void __launch_bounds__(1024) local_order_kernel(const unsigned* __restrict__ est,
-                                                           const unsigned* __restrict__ est2, int s,
-                                                           int* __restrict__ order, unsigned* __restrict__ est_min) {
-    __shared__ int cnt[33];
-    if (threadIdx.x < 33) cnt[threadIdx.x] = 0;
+// Members by decreasing estimate, four steps per power of two (a counting sort in one CTA; the order
+// within a class is arbitrary).
+__global__ void __launch_bounds__(1024) local_order_kernel(const unsigned* __restrict__ est, int s,
+                                                           int* __restrict__ order) {
+    __shared__ int cnt[128];
+    if (threadIdx.x < 128) cnt[threadIdx.x] = 0;
     __syncthreads();
-    for (int m = threadIdx.x; m < s; m += blockDim.x) {
-        const unsigned a = est[m], b = est2[m], e = b < a ? b : a;
-        est_min[m] = e;
-        atomicAdd(&cnt[__clz(e)], 1);
-    }
+    auto cls = [&](unsigned e) { return 4 * __clz(e) + (3 - (int)((e << __clz(e)) >> 29 & 3u)); };
+    for (int m = threadIdx.x; m < s; m += blockDim.x) atomicAdd(&cnt[cls(est[m] | 1u)], 1);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int c = 0; c < 33; ++c) {
-            const int x = cnt[c];
-            cnt[c] = acc;
-            acc += x;
+    if (threadIdx.x < 32) {  // exclusive scan of the 128 classes
+        int c[4], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            c[i] = sum;
+            sum += cnt[4 * threadIdx.x + i];
         }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((int)threadIdx.x >= o) incl += x;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) cnt[4 * threadIdx.x + i] = incl - sum + c[i];
     }
     __syncthreads();
-    for (int m = threadIdx.x; m < s; m += blockDim.x) {
-        const unsigned e = est_min[m];
-        order[atomicAdd(&cnt[__clz(e)], 1)] = m | (est2[m] < est[m] ? (1 << 30) : 0);
-    }
+    for (int m = threadIdx.x; m < s; m += blockDim.x) order[atomicAdd(&cnt[cls(est[m] | 1u)], 1)] = m;
 }
 
 // One CTA per member, labels in a global scratch slice per CTA.
@@ -482,7 +475,7 @@ __global__ void __launch_bounds__(1024) cc_global_kernel(GraphArgs g, const int*
     __shared__ long long red[32];
     __shared__ int sh_root;
     const int i = member_base + blockIdx.x;
-    member_pc<kVar>(labels + (size_t)blockIdx.x * g.n, g, pop + (size_t)i * k, k, i, &fit[i], status, red, &sh_root);
+    member_pc<kVar>(labels + (size_t)blockIdx.x * g.n, g, pop + (size_t)i * k, k, &fit[i], status, red, &sh_root);
 }
 
 // Forest-piece kernel: a persistent CTA of kPieceTeams teams of kPieceThreads threads per SM.
@@ -572,8 +565,7 @@ __global__ void __launch_bounds__(1024) piece_order_kernel(const unsigned* __res
     }
 }
 
-// The deferred members, with the cut-local TREE kernel (which runs the full pipeline for members
-// estimated to list over a quarter of the nodes): CTAs stride over list[0 .. *count).
+// The deferred members, with the cut-local TREE kernel: CTAs stride over list[0 .. *count).
 template <int kVar>
 __global__ void __launch_bounds__(1024) cc_list_kernel(GraphArgs g, const int* __restrict__ pop, int k,
                                                        long long* __restrict__ fit, int* status,
@@ -583,45 +575,74 @@ __global__ void __launch_bounds__(1024) cc_list_kernel(GraphArgs g, const int* _
     __shared__ int sh_root;
     const int cnt = *count;
     for (int x = blockIdx.x; x < cnt; x += gridDim.x) {
-        const int e = list[x];
-        const int i = e & 0x3FFFFFFF;
-        member_pc<kVar>(smem_lab, g, pop + (size_t)i * k, k, i, &fit[i], status, red, &sh_root, (e >> 30) & 1);
+        const int i = list[x] & 0x3FFFFFFF;
+        member_pc<kVar>(smem_lab, g, pop + (size_t)i * k, k, &fit[i], status, red, &sh_root);
         __syncthreads();  // the shared memory is reused by the next member
     }
 }
 
-template <int kVar>
-int launch_variant(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, int k, long long* f,
-                   cudaStream_t st, int* kernels = nullptr, const unsigned* est_in = nullptr) {
-    const int n = ga.n;
-    const size_t lab_bytes = kVar == V_TREE16    ? gapa_dev::tree16_smem_bytes(n)
-                             : kVar == V_TREE16L ? gapa_dev::tree16l_smem_bytes(n, (size_t)ga.list_bytes)
-                                                 : (size_t)n * 4;
-    if (lab_bytes <= c->fit_smem_max) {
-        const int* order = nullptr;
-        unsigned* est_min = nullptr;
-        if (kVar == V_TREE16L && s > 1 && s <= kOrderCap) {
-            // estimates under both forests (precomputed by the operator kernel, or here), then the order
-            unsigned* e1 = gapa_estimate_buffer(c);
-            unsigned* e2 = e1 + kOrderCap;
-            est_min = e2 + kOrderCap;
-            if (!est_in) {
-                const bool alt = c->g.has_alt;
-                local_cost_kernel<<<s, 128, 0, st>>>(pop, k, n, c->g.cut, alt ? c->g.alt.cut : nullptr, e1, e2);
-                if (kernels) *kernels += 1;
-            }
-            const unsigned* a = est_in ? est_in : e1;
-            local_order_kernel<<<1, 1024, 0, st>>>(a, a + kOrderCap, s, c->g.order, est_min);
-            order = c->g.order;
+// Members per SM of the cut-local kernel, its threads per member and its list region: as many members as
+// shared memory holds with lists of n / 2 entries, sharing the SM's 2048 threads, but no more than the
+// population spreads over the SMs, and no more than 256 (512) threads up to 1024 (2048) nodes.  Measured at
+// n = 20000 (1023 members of 1000 genes, random generation / hub-heavy fitness, whole call): three of 672
+// threads 68 / 85 us, three of 512 66 / 93; four of 512 hold lists of n / 3 entries only, and hub-heavy members
+// outgrow them.  80 members at n = 5009: 25 us with 1024 threads, 33 with 512.
+struct LocalShape {
+    int per_sm, threads, list_bytes;
+};
+
+LocalShape local_shape(const gapa_ctx* c, int s) {
+    const int n = c->g.n;
+    const size_t bm = gapa_dev::tree16l_bitmap_bytes(n), fixed = gapa_dev::tree16l_smem_bytes(n, 0);
+    const size_t least = std::max(gapa_dev::tree16l_min_list_bytes(n, c->g.mean_deg_x16), bm + (((size_t)n + 15) & ~(size_t)15));
+    const size_t most = bm + (((size_t)n * 2 + 1024 + 15) & ~(size_t)15);
+    int m = std::max(1, std::min(8, (s + c->num_sms - 1) / c->num_sms));
+    for (;; --m) {
+        const size_t block = c->smem_per_sm / (size_t)m, other = c->smem_reserved + 1024;
+        const size_t room = std::min(block > other ? block - other : 0, c->fit_smem_max);
+        if (m == 1 || room >= fixed + least) {
+            const size_t list = std::min(std::max(least, most), (room - fixed) & ~(size_t)15);
+            return LocalShape{m, std::min(n <= 1024 ? 256 : n <= 2048 ? 512 : 1024, (2048 / m) & ~31), (int)list};
+        }
+    }
+}
+
+// The cut-local kernel: members costliest first where not all of them run at once (estimates precomputed by
+// the operator kernel, or here; in order, the calls above take 70 and 97 us).
+int launch_local(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, int k, long long* f, cudaStream_t st,
+                 int* kernels, const unsigned* est_in) {
+    const LocalShape shape = local_shape(c, s);
+    const int* order = nullptr;
+    if (s > shape.per_sm * c->num_sms && s <= kOrderCap) {
+        unsigned* e1 = gapa_estimate_buffer(c);
+        if (!est_in) {
+            local_cost_kernel<<<s, 128, 0, st>>>(pop, k, c->g.n, c->g.lc.cost, nullptr, e1, e1 + kOrderCap);
             if (kernels) *kernels += 1;
         }
-        GraphArgs gl = ga;
-        gl.est = est_min;
-        cc_smem_kernel<kVar><<<s, smem_block_for(n), lab_bytes, st>>>(gl, pop, k, f, c->status, order);
+        const unsigned* a = est_in ? est_in : e1;
+        local_order_kernel<<<1, 1024, 0, st>>>(a, s, c->g.order);
+        order = c->g.order;
+        if (kernels) *kernels += 1;
+    }
+    GraphArgs gl = ga;
+    gl.list_bytes = shape.list_bytes;
+    cc_local_kernel<<<s, shape.threads, gapa_dev::tree16l_smem_bytes(ga.n, (size_t)shape.list_bytes), st>>>(
+        gl, pop, k, f, c->status, order);
+    GAPA_CUDA(cudaGetLastError());
+    return GAPA_OK;
+}
+
+template <int kVar>
+int launch_variant(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, int k, long long* f,
+                   cudaStream_t st) {
+    const int n = ga.n;
+    const size_t lab_bytes = kVar == V_TREE16 ? gapa_dev::tree32_smem_bytes(n) : (size_t)n * 4;
+    if (lab_bytes <= c->fit_smem_max) {
+        cc_smem_kernel<kVar><<<s, smem_block_for(n), lab_bytes, st>>>(ga, pop, k, f, c->status, nullptr);
         GAPA_CUDA(cudaGetLastError());
         return GAPA_OK;
     }
-    if constexpr (kVar == V_TREE16 || kVar == V_TREE16L) {
+    if constexpr (kVar == V_TREE16) {
         // 16-bit ids are chosen at upload only when the labels fit in shared memory
         return gapa_fail(GAPA_ERR_STATE, "16-bit tree labels need shared memory");
     } else {
@@ -692,9 +713,8 @@ int launch_piece(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, in
     const size_t parents = gapa_dev::piece_parents_bytes(n);
     const size_t avail = c->piece_smem_max > parents ? c->piece_smem_max - parents : 0;
     const gapa_dev::PieceLayout L = gapa_dev::piece_layout(n, k, kPieceThreads, avail / kPieceTeams);
-    const size_t lab_bytes = gapa_dev::tree16l_smem_bytes(n, (size_t)ga.list_bytes);
-    if (L.pcap < 512 || s < 2 || s > kOrderCap || lab_bytes > c->fit_smem_max)
-        return launch_variant<V_TREE16L>(c, ga, pop, s, k, f, st, kernels, est_in);
+    const LocalShape shape = local_shape(c, s);
+    if (L.pcap < 512 || s < 2 || s > kOrderCap) return launch_local(c, ga, pop, s, k, f, st, kernels, nullptr);
     unsigned* e1 = gapa_estimate_buffer(c);
     unsigned* e2 = e1 + kOrderCap;
     unsigned* est_min = e2 + kOrderCap;
@@ -716,8 +736,9 @@ int launch_piece(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, in
                                                                        ctl);
     GAPA_CUDA(cudaGetLastError());
     GraphArgs gl = ga;
-    gl.est = est_min;
-    cc_list_kernel<V_TREE16L><<<std::min(s, 2 * c->num_sms), smem_block_for(n), lab_bytes, st>>>(gl, pop, k, f,
+    gl.list_bytes = shape.list_bytes;
+    cc_list_kernel<V_TREE16L><<<std::min(s, 2 * c->num_sms), shape.threads,
+                                gapa_dev::tree16l_smem_bytes(n, (size_t)shape.list_bytes), st>>>(gl, pop, k, f,
                                                                                                c->status, defer, ctl);
     GAPA_CUDA(cudaGetLastError());
     if (kernels) *kernels += 3;
@@ -751,8 +772,6 @@ int gapa_fitness_prepare(gapa_ctx* c, int s) {
     return gapa_reserve((void**)&c->labels, &c->labels_cap, wave * (size_t)c->g.n, sizeof(int));
 }
 
-int gapa_fitness_block_for(int n) { return smem_block_for(n); }
-
 namespace {
 // Read-bandwidth probe: 16-byte loads over the buffer, grid-strided, four in
 // flight per thread; one word per CTA keeps the loads live.
@@ -783,25 +802,35 @@ int gapa_launch_read_probe(const void* buf, size_t bytes, int passes, int grid, 
     return GAPA_OK;
 }
 
-// AUTO picks the cut-local kernel above this many nodes: on smaller graphs the full pipeline is as
-// fast or faster (whole 100-generation runs: 40.5k against 34.0k generations/s at n = 1000, even at
-// n = 2000, 1.12-1.31 x for the cut-local kernel from n = 4000 to 12000)
-static constexpr int kLocalAutoMinNodes = 2049;
-
-static bool local_selected(const gapa_ctx* c) {
-    return c->g.packed16 && c->g.local_list_bytes > 0 &&
-           ((c->fitness_variant == GAPA_FITNESS_AUTO && c->g.n >= kLocalAutoMinNodes) ||
-            c->fitness_variant == GAPA_FITNESS_TREE_LOCAL);
+bool gapa_fitness_local(const gapa_ctx* c) {
+    const DeviceGraph& g = c->g;
+    // AUTO: not where most deletions leave much apart (mean degree below 3: trees, sparse random graphs), nor
+    // on small graphs of mean degree below 5.  Whole calls, 100 members of n / 20 genes (random and hub-heavy),
+    // cut-local against full pipeline, us: tree of 6000 nodes 42 / 17 and 41 / 17; degree 2.7, n = 6000: 28 / 33
+    // and 38 / 33, n = 1500: 24 / 19 and 29 / 19; degree 4, n = 700: 16 / 12 and 26 / 15, n = 3000: 19 / 23 and
+    // 24 / 26, n = 12000: 35 / 36 and 50 / 46; degree 6, n = 1500: 16 / 20 and 22 / 29, n = 12000: 21 / 55 and
+    // 43 / 57.
+    const bool sparse = g.mean_deg_x16 < 48 || (gapa_dev::tree16l_sparse(g.mean_deg_x16) && g.n <= 2048);
+    return g.packed16 && g.lc.par && (c->fitness_variant == GAPA_FITNESS_TREE_LOCAL ||
+                                      (c->fitness_variant == GAPA_FITNESS_AUTO && !sparse));
 }
+static bool local_selected(const gapa_ctx* c) { return gapa_fitness_local(c); }
 
 // The forest-piece kernel: by request only (it needs the cut-local kernel's forests and cost tables).
 static bool piece_selected(const gapa_ctx* c) {
-    return c->g.packed16 && c->g.local_list_bytes > 0 && c->g.sz && c->fitness_variant == GAPA_FITNESS_PIECE;
+    return c->g.packed16 && c->g.lc.par && c->g.sz && c->fitness_variant == GAPA_FITNESS_PIECE;
 }
 
 bool gapa_fitness_uses_estimates(const gapa_ctx* c, int s) {
-    return (local_selected(c) || piece_selected(c)) && s > 1 && s <= kOrderCap && c->genes == GAPA_GENES_NODES &&
+    return (local_selected(c) ? s > local_shape(c, s).per_sm * c->num_sms : piece_selected(c) && s > 1) &&
+           s <= kOrderCap && c->genes == GAPA_GENES_NODES &&
            (c->objective == GAPA_OBJECTIVE_PC || c->objective == GAPA_OBJECTIVE_MCN);
+}
+
+void gapa_estimate_tables(const gapa_ctx* c, const int** first, const int** second) {
+    const bool piece = piece_selected(c);
+    *first = piece ? c->g.cut : c->g.lc.cost;
+    *second = piece && c->g.has_alt ? c->g.alt.cut : nullptr;
 }
 
 unsigned* gapa_estimate_buffer(gapa_ctx* c) { return reinterpret_cast<unsigned*>(c->g.order + kOrderCap); }
@@ -831,12 +860,8 @@ int gapa_launch_fitness(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* 
     ga.join_mode = c->fitness_variant == GAPA_FITNESS_TREE_JOIN ? 1 : c->fitness_variant == GAPA_FITNESS_TREE_SCAN ? 2 : 0;
     ga.mean_deg_x16 = c->g.mean_deg_x16;
     ga.objective = c->objective;
-    ga.kids = c->g.kids;
-    ga.roots = c->g.roots;
-    ga.num_roots = c->g.num_roots;
-    ga.list_bytes = c->g.local_list_bytes;
-    ga.est = nullptr;
-    ga.alt = c->g.alt;
+    ga.lc = c->g.lc;
+    ga.list_bytes = 0;
     if (c->objective == GAPA_OBJECTIVE_SIXDST_PC || c->objective == GAPA_OBJECTIVE_SIXDST_MCN) {
         if (c->genes != GAPA_GENES_NODES) return gapa_fail(GAPA_ERR_INVALID_ARG, "SixDST objectives take node genes");
         return gapa_launch_fitness_sixdst(c, pop, s, k, fit, st, &prof.kernels);
@@ -860,7 +885,7 @@ int gapa_launch_fitness(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* 
             if (c->g.packed16) {
                 if (piece_selected(c) && c->objective <= GAPA_OBJECTIVE_MCN)
                     return launch_piece(c, ga, pop, s, k, f, st, &prof.kernels, est);
-                if (local_selected(c)) return launch_variant<V_TREE16L>(c, ga, pop, s, k, f, st, &prof.kernels, est);
+                if (local_selected(c)) return launch_local(c, ga, pop, s, k, f, st, &prof.kernels, est);
                 return launch_variant<V_TREE16>(c, ga, pop, s, k, f, st);
             }
             if ((size_t)n * 4 <= c->fit_smem_max) return launch_variant<V_TREE32>(c, ga, pop, s, k, f, st);
@@ -873,7 +898,7 @@ int gapa_fitness_kernels_init(gapa_ctx* c) {
     int rc = gapa_set_smem_limit((const void*)cc_smem_kernel<V_EDGES>, c->smem_optin, &c->fit_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_smem_kernel<V_SAMPLED>, c->smem_optin, &c->fit_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_smem_kernel<V_TREE16>, c->smem_optin, &c->fit_smem_max);
-    if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_smem_kernel<V_TREE16L>, c->smem_optin, &c->fit_smem_max);
+    if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_local_kernel, c->smem_optin, &c->fit_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_list_kernel<V_TREE16L>, c->smem_optin, &c->fit_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_piece_kernel, c->smem_optin, &c->piece_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_smem_kernel<V_TREE32>, c->smem_optin, &c->fit_smem_max);
@@ -1026,39 +1051,21 @@ __global__ void __launch_bounds__(1024, 1) fitness_batched_kernel(const BatchDes
         if (team < q.cnt) {
             const gapa_dev::Team tm{(int)threadIdx.x - team * T, T, 1 + team};
             const unsigned slice = (smem_bytes / (unsigned)q.teams) & ~15u;
-            int* lab = reinterpret_cast<int*>(smem + (size_t)team * slice);
+            gapa_dev::lab_t* lab = reinterpret_cast<gapa_dev::lab_t*>(smem + (size_t)team * slice);
             const gapa_dev::Tree16Graph g{bd.n,        bd.perm,      bd.palt,        bd.lo_ptr,   bd.lo_col,
                                           bd.nontree,  bd.num_nontree, bd.fptr,      bd.fcol16,   0,
-                                          bd.mean_deg_x16, bd.objective, bd.tparent, bd.kids,     bd.roots,
-                                          bd.num_roots, bd.list_bytes};
+                                          bd.mean_deg_x16, bd.objective, bd.lc,      bd.list_bytes,
+                                          gapa_dev::tree16l_tops_max(bd.n, bd.mean_deg_x16)};
             const int member = q.i0 + team;
             const int* genes = bd.pop[buf] + (size_t)member * bd.p.k;
             long long* out = reinterpret_cast<long long*>(bd.fit[buf]) + member;
-            // the cut-local kernel with the operator kernels' estimates: the cheaper forest, or the
-            // full pipeline for a member expected to shatter both
-            bool local = bd.list_bytes > 0, alt = false;
-            if (local && bd.p.est_out) {
-                const unsigned e1 = bd.p.est_out[member], e2 = bd.p.est_out[bd.p.est_stride + member];
-                const unsigned e = e2 < e1 ? e2 : e1;
-                if (e > (unsigned)(bd.n / 4)) local = false;
-                alt = e2 < e1 && bd.alt.perm != nullptr;
-            }
-            unsigned* region = reinterpret_cast<unsigned*>(lab + gapa_dev::tree16l_lab_ints(bd.n));
-            int* scal = reinterpret_cast<int*>(region) + bd.list_bytes / 4;
-            if (local && alt) {
-                const DeviceForest& a = bd.alt;
-                const gapa_dev::Tree16Graph tb{bd.n,         a.perm,          a.palt,          a.lo_ptr,
-                                               a.lo_col,     a.nontree,       a.num_nontree,   a.fptr,
-                                               a.fcol16,     0,               bd.mean_deg_x16, bd.objective,
-                                               a.tparent,    a.kids,          a.roots,         a.num_roots,
-                                               bd.list_bytes};
-                gapa_dev::tree16_member_local(tm, lab, region, scal, tb, genes, bd.p.k, out, red[team], status);
-            } else if (local) {
-                gapa_dev::tree16_member_local(tm, lab, region, scal, g, genes, bd.p.k, out, red[team], status);
-            } else {
-                gapa_dev::tree16_member(tm, lab, reinterpret_cast<unsigned*>(lab + bd.n), g, genes, bd.p.k, out,
-                                        red[team], status);
-            }
+            unsigned* region = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(lab) + gapa_dev::tree16_lab_bytes(bd.n));
+            if (bd.list_bytes > 0)
+                gapa_dev::tree16_member_local(tm, lab, region, reinterpret_cast<int*>(region) + bd.list_bytes / 4, g,
+                                              genes, bd.p.k, out, red[team], status);
+            else
+                gapa_dev::tree32_member(tm, reinterpret_cast<int*>(lab), reinterpret_cast<unsigned*>(lab) + bd.n, g,
+                                        genes, bd.p.k, out, red[team], status);
         }
         __syncthreads();
     }

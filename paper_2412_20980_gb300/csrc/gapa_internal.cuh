@@ -91,7 +91,7 @@ __device__ __forceinline__ int uniform_below(uint32_t x, int n) { return (int)__
 // ---------------------------------------------------------------------------
 // A second spanning forest of a graph with n <= 65536, in its own numbering
 // (parents precede children; a node's parent is its lowest-numbered
-// neighbour when that one is lower): the arrays of the TREE kernels.
+// neighbour when that one is lower), for the forest-piece kernel.
 struct DeviceForest {
     int* perm = nullptr;             // [n] original id -> number
     int* tparent = nullptr;          // [n rounded up to 4]
@@ -144,6 +144,20 @@ struct SparseForest {
 };
 constexpr int kSpForests = 4;
 
+// Tables of the cut-local TREE kernel (tree16.cuh), 16-bit numbers of the BFS forest (0xFFFF: none).
+struct CutTables {
+    unsigned short* par = nullptr;  // [n rounded up to 8] tree parent (roots: itself)
+    uint2* gene = nullptr;          // by original id: number | first child << 16, children | (single node) << 16
+    uint2* lower = nullptr;         // by number: the second to fourth and the last of its lower-numbered neighbours
+    uint2* higher = nullptr;        // by number: its four higher-numbered neighbours of highest degree among those
+                                    //     that are not its tree children
+    unsigned short* near = nullptr; // by number: its first eight neighbours in the adjacency's order (0xFFFF: fewer)
+    int* roots = nullptr;           // BFS number of the root of every component of two nodes or more
+    int num_roots = 0;
+    int singles = 0;                // single-node components
+    int* cost = nullptr;            // by original id: children + 1 (the member cost estimate sums it)
+};
+
 struct DeviceGraph {
     int n = 0;
     long long nnz = 0;        // arcs = 2E
@@ -162,13 +176,13 @@ struct DeviceGraph {
                                 //     where children have consecutive numbers)
     int* roots = nullptr;       // [num_roots] BFS number of every component's root
     int num_roots = 0;
-    int local_list_bytes = 0;   // list region of the cut-local TREE kernel (0: that kernel does not fit)
+    CutTables lc;               // cut-local TREE kernel (lc.par null: not on this graph)
     int* cut = nullptr;         // [n] per original node id: nodes below those of its tree children that
                                 //     have no other lower neighbour (deleting it alone cuts them off)
     int* order = nullptr;       // [5 * kOrderCap + 16] the members, costliest first (bit 30: use `alt`), then
                                 //     their cost estimates under this forest, under `alt`, and the lower,
                                 //     then the members deferred by the forest-piece kernel and their count
-    DeviceForest alt;           // the forest numbered with the top hubs last (cut-local kernel only)
+    DeviceForest alt;           // the forest numbered with the top hubs last (forest-piece kernel only)
     // forest-piece kernel, per forest: the subtree size of every node, its position in a preorder
     // walk (children in ascending order, roots in ascending order; a subtree is the interval
     // [pre, pre + sz)), the node at each preorder position, the smallest root of every node's
@@ -350,14 +364,9 @@ struct BatchDesc {
     int mean_deg_x16;
     int objective;       // GAPA_OBJECTIVE_*
     int teams;           // members per CTA in the batched fitness kernel (1, 2, 4 or 8)
-    // cut-local TREE kernel (tree16_member_local): list_bytes > 0 when each team's slice holds it;
-    // the members' cost estimates come from the operator kernels through p.est_out
-    const int* tparent;
-    const int4* kids;
-    const int* roots;
-    int num_roots;
+    // cut-local TREE kernel (tree16_member_local): list_bytes > 0 when each team's slice holds it
+    CutTables lc;
     int list_bytes;
-    DeviceForest alt;    // the second forest (alt.perm null: none)
 };
 
 // A packet of the batched fitness work queue: members i0 .. i0+cnt-1 of instance b.
@@ -370,8 +379,10 @@ int gapa_launch_fitness(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* 
 // True when gapa_launch_fitness runs the cut-local TREE kernel on this context (which then uses
 // per-member cost estimates; callers that produce the rows may pass them precomputed).
 bool gapa_fitness_uses_estimates(const gapa_ctx* c, int s);
-// Threads of the one-member-per-CTA fitness kernels for a graph of n nodes.
-int gapa_fitness_block_for(int n);
+// Whether the context's setting takes the cut-local TREE kernel on its graph.
+bool gapa_fitness_local(const gapa_ctx* c);
+// The cost tables that the operator kernels sum over a row's genes for that kernel's estimates.
+void gapa_estimate_tables(const gapa_ctx* c, const int** first, const int** second);
 // Device buffer of 2 * kOrderCap cost estimates owned by the graph (valid when the above is true):
 // row m's estimate under the first forest at [m], under the second at [kOrderCap + m] (0xFFFFFFFF
 // when the graph has no second forest).
