@@ -532,7 +532,6 @@ int ensure_variant_scratch(gapa_ctx* c, const gapa_config* cfg) {
     if (rc == GAPA_OK && (cfg->flags & GAPA_FLAG_MU_PLUS_LAMBDA)) {
         rc = gapa_reserve((void**)&c->kids, &c->kids_cap, (size_t)cfg->lambda * cfg->k, 4);
         if (rc == GAPA_OK) rc = gapa_reserve((void**)&c->kfit, &c->kfit_cap, (size_t)cfg->lambda, 8);
-        if (rc == GAPA_OK) rc = gapa_reserve((void**)&c->src, &c->src_cap, (size_t)cfg->pop, 4);
     }
     if (rc == GAPA_OK)
         rc = gapa_fitness_prepare(c, (cfg->flags & GAPA_FLAG_MU_PLUS_LAMBDA) ? std::max(cfg->pop, cfg->lambda)
@@ -564,8 +563,7 @@ int enqueue_generation(gapa_ctx* c, const GaParams& p0, int lambda, const int32_
         rc = gapa_launch_children(c, p, lambda, pop_in, fit_in, c->kids, st);
         if (rc == GAPA_OK) rc = gapa_launch_fitness(c, c->kids, lambda, p.k, c->kfit, st, est);
         if (rc == GAPA_OK)
-            rc = gapa_launch_mpl_replace(c, p.s, lambda, p.k, pop_in, fit_in, c->kids, c->kfit, c->src, pop_out,
-                                         fit_out, st);
+            rc = gapa_launch_mpl_replace(c, p.s, lambda, p.k, pop_in, fit_in, c->kids, c->kfit, pop_out, fit_out, st);
         return rc;
     }
     rc = gapa_launch_offspring(c, p, pop_in, fit_in, pop_out, fit_out, st);
@@ -741,7 +739,7 @@ void gapa_destroy(gapa_ctx* c) {
     cudaFree(c->status);
     cudaFree(c->labels);
     cudaFree(c->ig_aux);
-    cudaFree(c->sp_scratch);
+    gapa_sparse_release(c);
     cudaFree(c->sp_order);
     cudaFree(c->sdst_buf);
     for (auto p : c->stage_pop) cudaFree(p);
@@ -752,7 +750,6 @@ void gapa_destroy(gapa_ctx* c) {
     cudaFree(c->kids);
     cudaFree(c->kfit);
     cudaFree(c->cum);
-    cudaFree(c->src);
     for (auto& t : c->timed) {
         cudaEventDestroy(t.a);
         cudaEventDestroy(t.b);

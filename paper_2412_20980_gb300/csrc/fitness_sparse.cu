@@ -104,8 +104,8 @@ __device__ __forceinline__ unsigned ldcg(const unsigned* p) { return __ldcg(p); 
 __device__ __forceinline__ unsigned long long ldcg(const unsigned long long* p) { return __ldcg(p); }
 
 __host__ __device__ __forceinline__ size_t sp_bitmap_bytes(int n) { return ((((size_t)n + 31) >> 5) * 4 + 15) & ~(size_t)15; }
-__host__ __device__ __forceinline__ size_t sp_smem_bytes(int n, int k) {
-    return sp_bitmap_bytes(n) + (((size_t)2 * k + 1) * 4 + 15) / 16 * 16 + (size_t)3 * kSpBlock * 4;
+__host__ __device__ __forceinline__ size_t sp_smem_bytes(int n, int k, int threads) {
+    return sp_bitmap_bytes(n) + (((size_t)2 * k + 1) * 4 + 15) / 16 * 16 + (size_t)3 * threads * 4;
 }
 
 // Class of value a (terminal + 1; 0 = R): the root's value r, with the links
@@ -182,31 +182,28 @@ struct SpCostArgs {
     int hub0, hub1;
 };
 
-__global__ void __launch_bounds__(128) sp_cost_kernel(const int* __restrict__ pop, int k, int n, SpCostArgs a,
-                                                      unsigned* __restrict__ est, int* __restrict__ forest) {
-    __shared__ unsigned long long part[4];
-    __shared__ int s_f;
-    const int m = blockIdx.x, t = threadIdx.x;
+__global__ void __launch_bounds__(1024) sp_cost_kernel(const int* __restrict__ pop, int k, int n, SpCostArgs a,
+                                                       unsigned* __restrict__ est, int* __restrict__ forest) {
+    __shared__ unsigned long long part[32];
+    const int m = blockIdx.x, t = threadIdx.x, T = blockDim.x;
     const int* genes = pop + (size_t)m * k;
     int h0 = 0, h1 = 0;
-    for (int j = t; j < k; j += 128) {
+#pragma unroll 4
+    for (int j = t; j < k; j += T) {
         const int d = __ldg(&genes[j]);
         h0 |= d == a.hub0;
         h1 |= d == a.hub1;
     }
     h0 = __syncthreads_or(h0);
     h1 = __syncthreads_or(h1);
-    if (t == 0) {
-        int f = 0;
-        if (h0 && h1 && a.cost[2]) f = 2;
-        else if (h0 && a.cost[1]) f = 1;
-        else if (h1 && a.cost[3]) f = 3;
-        s_f = f;
-    }
-    __syncthreads();
-    const int* cost = a.cost[s_f];
+    int f = 0;
+    if (h0 && h1 && a.cost[2]) f = 2;
+    else if (h0 && a.cost[1]) f = 1;
+    else if (h1 && a.cost[3]) f = 3;
+    const int* cost = a.cost[f];
     unsigned long long c = 0;
-    for (int j = t; j < k; j += 128) {
+#pragma unroll 4
+    for (int j = t; j < k; j += T) {
         const int d = __ldg(&genes[j]);
         if ((unsigned)d < (unsigned)n) c += (unsigned)__ldg(&cost[d]);
     }
@@ -214,9 +211,10 @@ __global__ void __launch_bounds__(128) sp_cost_kernel(const int* __restrict__ po
     if ((t & 31) == 0) part[t >> 5] = c;
     __syncthreads();
     if (t == 0) {
-        const unsigned long long tot = part[0] + part[1] + part[2] + part[3];
+        unsigned long long tot = 0;
+        for (int w = 0; w < T >> 5; ++w) tot += part[w];
         est[m] = tot > 0xFFFFFFFFull ? 0xFFFFFFFFu : (unsigned)tot;
-        forest[m] = s_f;
+        forest[m] = f;
     }
 }
 
@@ -244,8 +242,8 @@ __global__ void __launch_bounds__(1024) sp_order_kernel(const unsigned* __restri
         order[atomicAdd(&cnt[__clz(est[m])], 1)] = m | (forest[m] << kSpForestShift);
 }
 
-template <typename Col>
-__global__ void __launch_bounds__(kSpBlock, 1) cc_sparse_kernel(const __grid_constant__ SpGraphs<Col> gs, SpSlot base,
+template <typename Col, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_sparse_kernel(const __grid_constant__ SpGraphs<Col> gs, SpSlot base,
                                                                size_t stride, const int* __restrict__ pop, int s,
                                                                int k, long long* __restrict__ fit, int* head,
                                                                int* status, const int* __restrict__ order) {
@@ -258,7 +256,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) cc_sparse_kernel(const __grid_con
     unsigned* dead = reinterpret_cast<unsigned*>(sp_smem);
     int* D = reinterpret_cast<int*>(sp_smem + sp_bitmap_bytes(n));
     int* Doff = D + k;  // nd + 1 entries
-    int* s_off = reinterpret_cast<int*>(sp_smem + sp_smem_bytes(n, k) - (size_t)3 * kSpBlock * 4);
+    int* s_off = reinterpret_cast<int*>(sp_smem + sp_smem_bytes(n, k, T) - (size_t)3 * T * 4);
     int* s_first = s_off + T;
     int* s_val = s_first + T;
     int* ws = reinterpret_cast<int*>(red);
@@ -766,21 +764,57 @@ SpGraphs<Col> sp_graphs(const gapa_ctx* c) {
 }  // namespace
 
 bool gapa_sparse_fits(const gapa_ctx* c, int k) {
-    return c->g.sp_nforests > 0 && c->sp_smem_max > 0 && sp_smem_bytes(c->g.n, k) <= c->sp_smem_max;
+    return c->g.sp_nforests > 0 && c->sp_smem_max > 0 && sp_smem_bytes(c->g.n, k, kSpBlock) <= c->sp_smem_max;
+}
+
+// Teams per SM and their threads: 1 x 1024, 2 x 512, 4 or 6 x 256 (the small teams' kernel is held to 42
+// registers), the most that leave every SM two rounds of members to balance, that shared memory holds and
+// that keep the scratch within 4 GB.  A member's phases wait at barriers and on scattered reads, so several
+// smaller teams cover each other; with a single round the largest member, now on fewer threads, is what the
+// call waits for (310 members of 2000 genes, n = 70000, BA(3): 139 us at 1 per SM, 167 at 2).  At 1 / 2 / 4
+// per SM: 620 members 227 / 183 / 283 us, 1300 members 416 / 300 / 294.  One (mu+lambda) generation with 2048
+// children (2000 genes, n = 100000, BA(3)), at 1 / 2 / 4 / 6: 706 / 529 / 510 / 472 us.
+constexpr int kSpTeams[4] = {1, 2, 4, 6}, kSpThreads[4] = {1024, 512, 256, 256};
+
+static int sp_shape(const gapa_ctx* c, int s, int k) {
+    int i = 3;
+    for (; i > 0; --i) {
+        const long long teams = (long long)kSpTeams[i] * c->num_sms;
+        if (s >= 2 * teams && (size_t)teams * c->g.n * 44 <= ((size_t)4 << 30) &&
+            kSpTeams[i] * (sp_smem_bytes(c->g.n, k, kSpThreads[i]) + c->smem_reserved + 1024) <= c->smem_per_sm)
+            break;
+    }
+    return i;
 }
 
 int gapa_sparse_init(gapa_ctx* c) {
-    int rc = gapa_set_smem_limit((const void*)cc_sparse_kernel<int>, c->smem_optin, &c->sp_smem_max);
-    size_t other = 0;
-    if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)cc_sparse_kernel<unsigned short>, c->smem_optin, &other);
-    if (other < c->sp_smem_max) c->sp_smem_max = other;
-    return rc;
+    const void* kernels[4] = {(const void*)cc_sparse_kernel<int, false>, (const void*)cc_sparse_kernel<unsigned short, false>,
+                              (const void*)cc_sparse_kernel<int, true>, (const void*)cc_sparse_kernel<unsigned short, true>};
+    for (int i = 0; i < 4; ++i) {
+        size_t dyn = 0;
+        const int rc = gapa_set_smem_limit(kernels[i], c->smem_optin, &dyn);
+        if (rc != GAPA_OK) return rc;
+        c->sp_smem_max = i == 0 ? dyn : std::min(c->sp_smem_max, dyn);
+    }
+    return GAPA_OK;
+}
+
+void gapa_sparse_release(gapa_ctx* c) {
+    cudaFree(c->sp_scratch);
+    c->sp_scratch = nullptr;
+    c->sp_scratch_cap = 0;
+    for (void*& old : c->sp_old) {
+        cudaFree(old);
+        old = nullptr;
+    }
 }
 
 // Scratch of the persistent CTAs: nine n-entry arrays per CTA (hops, classes,
 // counts, listed nodes, live tops, their hops, touched components: int32;
-// per-component sums and reference keys: int64), set to -1 / 0 once here and
-// left that way by every member.
+// per-component sums and reference keys: int64).  All but the lists are set to
+// -1 / 0 once here and left that way by every member.  A larger population may ask for more slices: the
+// smaller block then stays until the context or the graph goes, as captured work
+// may still point to it.
 int gapa_sparse_prepare(gapa_ctx* c, int s) {
     const int n = c->g.n;
     const size_t stride = ((size_t)n + 63) & ~(size_t)63;
@@ -789,28 +823,31 @@ int gapa_sparse_prepare(gapa_ctx* c, int s) {
         int rc = gapa_reserve((void**)&c->sp_order, &c->sp_order_cap, (size_t)3 * std::max(s, 1), sizeof(int));
         if (rc != GAPA_OK) return rc;
     }
-    if (c->sp_scratch && c->sp_stride == stride) return GAPA_OK;  // (also inside a stream capture)
-    const size_t smem = sp_smem_bytes(n, 0);
-    int per_sm = 0;
-    GAPA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cc_sparse_kernel<int>, kSpBlock, smem));
-    if (per_sm < 1) per_sm = 1;
-    const int slots = c->num_sms * per_sm;
+    const int slots = c->num_sms * kSpTeams[sp_shape(c, s, 0)];
+    if (c->sp_scratch && c->sp_stride == stride && c->sp_slots >= slots) return GAPA_OK;  // (also inside a stream capture)
     const size_t bytes = (size_t)slots * stride * (7 * 4 + 2 * 8) + 64;
-    cudaFree(c->sp_scratch);
-    c->sp_scratch = nullptr;
-    c->sp_scratch_cap = 0;
-    if (cudaMalloc(&c->sp_scratch, bytes) != cudaSuccess) {
+    if (c->sp_stride != stride) gapa_sparse_release(c);
+    void* block = nullptr;
+    if (cudaMalloc(&block, bytes) != cudaSuccess) {
         cudaGetLastError();
+        if (c->sp_scratch) return GAPA_OK;  // the smaller block serves
         return gapa_fail(GAPA_ERR_OOM, "sparse fitness scratch of %zu bytes", bytes);
     }
+    for (void*& old : c->sp_old)
+        if (!old) {
+            old = c->sp_scratch;
+            break;
+        }
+    c->sp_scratch = block;
     c->sp_scratch_cap = bytes;
     c->sp_stride = stride;
     c->sp_slots = slots;
     const size_t ints = (size_t)slots * stride;
     char* p = static_cast<char*>(c->sp_scratch);
-    // hop, cls = -1; cnt, list, tl, th, cl = 0; cacc, best = 0; the queue head last
-    GAPA_CUDA(cudaMemset(p, 0xFF, ints * 8));
-    GAPA_CUDA(cudaMemset(p + ints * 8, 0, ints * 20 + ints * 16 + 64));
+    // hop, cls = -1; cnt, cacc, best = 0 (the lists are read only as far as a member wrote them); the queue head last
+    GAPA_CUDA(cudaMemsetAsync(p, 0xFF, ints * 8));
+    GAPA_CUDA(cudaMemsetAsync(p + ints * 8, 0, ints * 4));
+    GAPA_CUDA(cudaMemsetAsync(p + ints * 28, 0, ints * 16 + 64));
     GAPA_CUDA(cudaDeviceSynchronize());
     return GAPA_OK;
 }
@@ -834,8 +871,10 @@ int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, in
     b.best = reinterpret_cast<unsigned long long*>(p + ints * 36);
     int* head = reinterpret_cast<int*>(p + ints * 44);
     GAPA_CUDA(cudaMemsetAsync(head, 0, sizeof(int), st));
-    const size_t smem = sp_smem_bytes(c->g.n, k);
-    const int grid = std::min(c->sp_slots, std::max(s, 1));
+    int shape = sp_shape(c, s, k);
+    while (shape > 0 && c->num_sms * kSpTeams[shape] > c->sp_slots) --shape;  // (a smaller block had to serve)
+    const int T = kSpThreads[shape], grid = std::min(c->num_sms * kSpTeams[shape], std::max(s, 1));
+    const size_t smem = sp_smem_bytes(c->g.n, k, T);
     // every member's forest and cost estimate, then the members costliest first
     unsigned* est = reinterpret_cast<unsigned*>(c->sp_order + s);
     int* forest = c->sp_order + 2 * (size_t)s;
@@ -843,16 +882,18 @@ int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, in
     for (int i = 0; i < kSpForests; ++i) ca.cost[i] = c->g.spf[i].kids ? c->g.spf[i].cost : nullptr;
     ca.hub0 = c->g.sp_hub[0];
     ca.hub1 = c->g.sp_hub[1];
-    sp_cost_kernel<<<s, 128, 0, st>>>(pop, k, c->g.n, ca, est, forest);
+    const int ct = k <= 1024 ? 128 : k <= 4096 ? 256 : 1024;  // about eight genes per thread
+    sp_cost_kernel<<<s, ct, 0, st>>>(pop, k, c->g.n, ca, est, forest);
     sp_order_kernel<<<1, 1024, 0, st>>>(est, forest, s, c->sp_order);
+    auto launch = [&](auto kernel, auto graphs) {
+        kernel<<<grid, T, smem, st>>>(graphs, b, c->sp_stride, pop, s, k, reinterpret_cast<long long*>(fit), head,
+                                      c->status, c->sp_order);
+    };
     if (c->g.packed16)
-        cc_sparse_kernel<unsigned short><<<grid, kSpBlock, smem, st>>>(sp_graphs<unsigned short>(c), b, c->sp_stride,
-                                                                        pop, s, k, reinterpret_cast<long long*>(fit),
-                                                                        head, c->status, c->sp_order);
+        launch(shape ? cc_sparse_kernel<unsigned short, true> : cc_sparse_kernel<unsigned short, false>,
+               sp_graphs<unsigned short>(c));
     else
-        cc_sparse_kernel<int><<<grid, kSpBlock, smem, st>>>(sp_graphs<int>(c), b, c->sp_stride, pop, s, k,
-                                                             reinterpret_cast<long long*>(fit), head, c->status,
-                                                             c->sp_order);
+        launch(shape ? cc_sparse_kernel<int, true> : cc_sparse_kernel<int, false>, sp_graphs<int>(c));
     GAPA_CUDA(cudaGetLastError());
     if (kernels) *kernels = 3;
     return GAPA_OK;

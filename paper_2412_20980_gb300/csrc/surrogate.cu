@@ -1668,8 +1668,7 @@ int gapa_run_surrogate(gapa_ctx* c, const gapa_config* cfg, gapa_surrogate* s, i
             GAPA_CUDA(cudaMemcpyAsync(diag_exact_host + diag_rows, c->kfit, (size_t)lam * 8, cudaMemcpyDeviceToHost, st));
             diag_rows += lam;
         }
-        rc2 = gapa_launch_mpl_replace(c, mu, lam, k, P[cur], F[cur], c->kids, c->kfit, c->src, P[cur ^ 1], F[cur ^ 1],
-                                      st);
+        rc2 = gapa_launch_mpl_replace(c, mu, lam, k, P[cur], F[cur], c->kids, c->kfit, P[cur ^ 1], F[cur ^ 1], st);
         if (rc2 == GAPA_OK) rc2 = gapa_launch_record(c, F[cur ^ 1], mu, c->run_gen, c->run_traj, c->run_best, st);
         // online training on the ring
         if (rc2 == GAPA_OK && s && ring_valid >= s->cfg.batch && s->cfg.train_steps > 0) {
