@@ -365,6 +365,7 @@ struct BatchDesc {
     // cut-local TREE kernel (tree16_member_local): list_bytes > 0 when each team's slice holds it
     CutTables lc;
     int list_bytes;
+    size_t set_off;      // best set's offset in the packed results
 };
 
 // A packet of the batched fitness work queue: members i0 .. i0+cnt-1 of instance b.

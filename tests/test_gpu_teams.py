@@ -1,4 +1,4 @@
-"""Small teams of the sparse kernel and the (mu+lambda) ranks against the oracle at the edges of their rules."""
+"""Small teams of the sparse kernel, the (mu+lambda) ranks and packed batch results against the oracle at the edges of their rules."""
 import numpy as np
 import pytest
 
@@ -51,3 +51,28 @@ def test_mu_plus_lambda_ranks_match_oracle(ctx, mu, lam, k):
     from test_gpu_ga import MPL, _gen_case
 
     _gen_case(ctx, synth.ba_graph(300, 2, 1), k, mu, 0.6, 0.05, 2, 9, MPL, 3, lam=lam)
+
+
+# one object over longer and shorter runs and other teams: results, trajectories and sets of every size
+@pytest.mark.parametrize("ks", [(0, 1, 31, 2000), (2999, 0, 0, 1)])
+def test_batch_results_of_repeated_runs_match_oracle(ks):
+    from paper_2412_20980_gb300 import Batch, Context, make_config
+
+    graphs = [synth.ba_graph(n, 3, 5) for n in (3000, 33, 64, 20011)]
+    ctxs, cfgs = [], []
+    for g, k in zip(graphs, ks):
+        ctxs.append(Context(0))
+        ctxs[-1].graph_upload(g.row_ptr, g.col)
+        cfgs.append(make_config(k=k, pop=6, tourn=2, pc=0.8, pm=0.1, seed=k))
+    bt = Batch(ctxs, cfgs)
+    for gens, teams in [(2, None), (5, None), (0, None), (4, [2, 8, 4, 1]), (4, [1, 1, 1, 1])]:
+        if teams:
+            bt.teams = teams
+        got = bt.run(gens)
+        for i, (g, cfg) in enumerate(zip(graphs, cfgs)):
+            want = oracle.run(g.row_ptr, g.col, k=cfg.k, pop=cfg.pop, gens=gens, tourn=cfg.tourn, pc_thr=cfg.pc_thr,
+                              pm_thr=cfg.pm_thr, seed=cfg.seed, nthreads=oracle.max_threads())
+            assert np.array_equal(got["traj"][i], want["traj"]), (gens, i)
+            assert got["best_fit"][i] == want["best_fit"], (gens, i)
+            assert np.array_equal(got["best_sets"][i], want["best_set"]), (gens, i)
+    bt.close()
