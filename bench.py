@@ -190,9 +190,9 @@ DEFAULT_TRAFFIC_SOURCES = ("fitness.cu", "tree16.cuh", "gapa_internal.cuh")
 
 
 KERNEL_TEXT = {
-    ("throughput", "auto"): "fitness phase: local_order_kernel + cc_smem_kernel<4> (cut-local TREE, two forests, "
+    ("throughput", "auto"): "fitness phase: local_order_kernel + cc_local_kernel (cut-local, 16-bit labels, "
                             "estimates written by the operator kernel)",
-    ("small", "auto"): "cc_smem_kernel (full TREE pipeline, shared-memory labels; n <= 2048)",
+    ("small", "auto"): "cc_local_kernel (cut-local, 16-bit labels, one CTA of 256 threads per member)",
     ("large", "auto"): "cc_sparse_kernel<int> (sparse: re-picked tops, hop chains, sampled terminal links, listed "
                        "pieces only; one persistent CTA per member)",
     ("large", "tree"): "ig_* kernels (interleaved global labels, 8 members per 32-byte sector)",
@@ -542,21 +542,17 @@ def run_gapa(args, env: Env, gs):
         # 1000-node graph is launch- and latency-bound, graded by generations per second
         fit_launches = 0
     if fit_launches and wl == "sixdst":
-        # tensor-bound: 3 dense products of n x n 0/1 matrices per evaluation ((A+I)^2, ^4, ^6)
-        flop = 3 * 2.0 * float(gs[0].n) ** 3
-        d = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
-            os.path.join(ROOT, "MEASURED_PEAKS.json")) else {"bf16_tflops": 1900.0}
-        peak = 2.0 * float(d["bf16_tflops"])
-        achieved = flop * fit_evals / (fit_ms / 1000.0) / 1e12
-        roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+        # bound by shared-memory gathers: 16 bytes per arc and node, 128-column strip and hop after the first
+        n_, hops = int(gs[0].n), 6
+        gather = (2 * int(gs[0].num_edges) + n_) * ((n_ + 127) // 128) * 16 * (hops - 1)
+        props = torch.cuda.get_device_properties(dev)
+        peak = props.multi_processor_count * 128 * 2.07  # GB/s
+        achieved = gather * fit_evals / (fit_ms / 1000.0) / 1e9
+        roofline = {"bound": "shared memory", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": None,
-                    "kernel": "sdst_gemm_t7_kernel (tcgen05.mma kind::f8f6f4 E4M3, operands loaded by "
-                              "cp.async.bulk.tensor in 128-byte swizzled boxes, producer and MMA threads split, "
-                              "256 x 256 tiles as two M = 128, N = 256 products, FP32 accumulators in TMEM)",
-                    "flop_per_eval": flop, "evals": fit_evals, "fitness_ms": fit_ms,
-                    "peak_source": "measured bf16 burst (MEASURED_PEAKS.json bf16_tflops) x 2, the FP8/BF16 nominal "
-                                   "ratio" if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else
-                                   "fallback 1.9 PFLOP/s bf16 x 2",
+                    "kernel": "sdst_bits_kernel (bit rows of 128 columns in shared memory, one gather per arc and hop)",
+                    "bytes_per_eval": gather, "evals": fit_evals, "fitness_ms": fit_ms,
+                    "peak_source": "nominal: 128 bytes per SM and clock at 2070 MHz",
                     "fitness_share_of_step": fit_ms / max(1e-9, total_ms)}
     elif fit_launches:
         beval = bytes_per_eval(gs[0].n, gs[0].num_edges, k)
