@@ -220,16 +220,39 @@ __global__ void __launch_bounds__(1024) sp_cost_kernel(const int* __restrict__ p
 
 // Members by decreasing estimate (a counting sort on the estimate's bit length; one CTA), so that
 // the persistent CTAs take the costliest members first and none starts late; entry = member |
-// forest << 28.
+// forest << 28.  Where the call may run in small teams, `slots` of them, *small says whether it does:
+// when the costliest member, on its share of an SM, is no more than its slot's share of the sum of
+// the estimates (else that member is what the call waits for; see sp_shape), and the members are light,
+// four tops a gene at the mean (two for random genes; heavier members fill their SM's scattered accesses).
 __global__ void __launch_bounds__(1024) sp_order_kernel(const unsigned* __restrict__ est,
                                                         const int* __restrict__ forest, int s,
-                                                        int* __restrict__ order) {
+                                                        int* __restrict__ order, int slots, int k, int* __restrict__ small) {
     __shared__ int cnt[33];
+    __shared__ unsigned long long sum;
+    __shared__ unsigned most;
     if (threadIdx.x < 33) cnt[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        sum = 0;
+        most = 0;
+    }
     __syncthreads();
-    for (int m = threadIdx.x; m < s; m += blockDim.x) atomicAdd(&cnt[__clz(est[m])], 1);
+    unsigned long long part = 0;
+    unsigned mx = 0;
+    for (int m = threadIdx.x; m < s; m += blockDim.x) {
+        const unsigned e = est[m];
+        atomicAdd(&cnt[__clz(e)], 1);
+        part += e;
+        mx = max(mx, e);
+    }
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&sum, part);
+        atomicMax(&most, mx);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
+        *small = (unsigned long long)most * (unsigned)slots <= sum && sum <= 4ull * (unsigned)k * (unsigned)s;
         int acc = 0;
         for (int c = 0; c < 33; ++c) {
             const int x = cnt[c];
@@ -246,7 +269,8 @@ template <typename Col, bool SMALL>
 __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_sparse_kernel(const __grid_constant__ SpGraphs<Col> gs, SpSlot base,
                                                                size_t stride, const int* __restrict__ pop, int s,
                                                                int k, long long* __restrict__ fit, int* head,
-                                                               int* status, const int* __restrict__ order) {
+                                                               int* status, const int* __restrict__ order, int either) {
+    if (either && (head[1] != 0) != SMALL) return;  // the other shape's launch takes the call
     extern __shared__ __align__(16) unsigned char sp_smem[];
     __shared__ long long red[32];
     __shared__ int s_member, s_forest, s_nd, s_nt, s_nterm, s_ncl, s_gdel, s_nlist;
@@ -773,7 +797,9 @@ bool gapa_sparse_fits(const gapa_ctx* c, int k) {
 // smaller teams cover each other; with a single round the largest member, now on fewer threads, is what the
 // call waits for (310 members of 2000 genes, n = 70000, BA(3): 139 us at 1 per SM, 167 at 2).  At 1 / 2 / 4
 // per SM: 620 members 227 / 183 / 283 us, 1300 members 416 / 300 / 294.  One (mu+lambda) generation with 2048
-// children (2000 genes, n = 100000, BA(3)), at 1 / 2 / 4 / 6: 706 / 529 / 510 / 472 us.
+// children (2000 genes, n = 100000, BA(3)), at 1 / 2 / 4 / 6: 706 / 529 / 510 / 472 us.  Members of uneven cost
+// (up to all genes among the hubs, n = 100000) go the other way, 2048 of them 3551 / 3620 / 4396 / 3872, 762 of
+// them 1421 / 1734 at 1 / 2: the order kernel keeps such calls at one member per SM.
 constexpr int kSpTeams[4] = {1, 2, 4, 6}, kSpThreads[4] = {1024, 512, 256, 256};
 
 static int sp_shape(const gapa_ctx* c, int s, int k) {
@@ -873,8 +899,6 @@ int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, in
     GAPA_CUDA(cudaMemsetAsync(head, 0, sizeof(int), st));
     int shape = sp_shape(c, s, k);
     while (shape > 0 && c->num_sms * kSpTeams[shape] > c->sp_slots) --shape;  // (a smaller block had to serve)
-    const int T = kSpThreads[shape], grid = std::min(c->num_sms * kSpTeams[shape], std::max(s, 1));
-    const size_t smem = sp_smem_bytes(c->g.n, k, T);
     // every member's forest and cost estimate, then the members costliest first
     unsigned* est = reinterpret_cast<unsigned*>(c->sp_order + s);
     int* forest = c->sp_order + 2 * (size_t)s;
@@ -884,17 +908,22 @@ int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, in
     ca.hub1 = c->g.sp_hub[1];
     const int ct = k <= 1024 ? 128 : k <= 4096 ? 256 : 1024;  // about eight genes per thread
     sp_cost_kernel<<<s, ct, 0, st>>>(pop, k, c->g.n, ca, est, forest);
-    sp_order_kernel<<<1, 1024, 0, st>>>(est, forest, s, c->sp_order);
-    auto launch = [&](auto kernel, auto graphs) {
-        kernel<<<grid, T, smem, st>>>(graphs, b, c->sp_stride, pop, s, k, reinterpret_cast<long long*>(fit), head,
-                                      c->status, c->sp_order);
+    sp_order_kernel<<<1, 1024, 0, st>>>(est, forest, s, c->sp_order, c->num_sms * kSpTeams[shape], k, head + 1);
+    // a call that may run in small teams launches both shapes, one of which returns at once (about 3 us)
+    auto launch = [&](auto kernel, auto graphs, int i) {
+        const int T = kSpThreads[i], grid = std::min(c->num_sms * kSpTeams[i], std::max(s, 1));
+        kernel<<<grid, T, sp_smem_bytes(c->g.n, k, T), st>>>(graphs, b, c->sp_stride, pop, s, k,
+                                                            reinterpret_cast<long long*>(fit), head, c->status,
+                                                            c->sp_order, shape > 0);
     };
-    if (c->g.packed16)
-        launch(shape ? cc_sparse_kernel<unsigned short, true> : cc_sparse_kernel<unsigned short, false>,
-               sp_graphs<unsigned short>(c));
-    else
-        launch(shape ? cc_sparse_kernel<int, true> : cc_sparse_kernel<int, false>, sp_graphs<int>(c));
+    if (c->g.packed16) {
+        if (shape) launch(cc_sparse_kernel<unsigned short, true>, sp_graphs<unsigned short>(c), shape);
+        launch(cc_sparse_kernel<unsigned short, false>, sp_graphs<unsigned short>(c), 0);
+    } else {
+        if (shape) launch(cc_sparse_kernel<int, true>, sp_graphs<int>(c), shape);
+        launch(cc_sparse_kernel<int, false>, sp_graphs<int>(c), 0);
+    }
     GAPA_CUDA(cudaGetLastError());
-    if (kernels) *kernels = 3;
+    if (kernels) *kernels = shape ? 4 : 3;
     return GAPA_OK;
 }
