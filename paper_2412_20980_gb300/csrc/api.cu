@@ -961,7 +961,7 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     g.num_nontree = (int)bf.nontree.size();
     g.mean_deg_x16 = n > 0 ? (int)((16 * nnz + n - 1) / n) : 0;
     // 16-bit ids only on the shared-memory path (labels + deleted-node bitmap)
-    // (the limit: 4 bytes per node and a bitmap within shared memory, n <= about 57,000)
+    // (the limit: 4 bytes per node, a bitmap and four scalars within a block's shared memory, n <= about 56,280)
     g.packed16 = n < gapa_dev::kDead16 && gapa_dev::tree32_smem_bytes(n) <= c->fit_smem_max;
     const size_t nt_bytes = (g.packed16 ? 4 : 8) * std::max<size_t>(bf.nontree.size(), 4);
     if (cudaMalloc(&g.perm, sizeof(int32_t) * (size_t)n) != cudaSuccess ||
@@ -988,7 +988,7 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
             else if (kids[p].x + kids[p].y != x) contiguous = false;
             kids[p].y += 1;
         }
-        if (contiguous && gapa_dev::tree16l_smem_bytes(n, gapa_dev::tree16l_min_list_bytes(n, g.mean_deg_x16)) <= c->fit_smem_max) {
+        if (contiguous && gapa_dev::local_admits(n, g.mean_deg_x16, c->fit_smem_max)) {
             const int lrc = upload_cut_tables(bf, rp, sorted, n, kids, g.lc);
             if (lrc != GAPA_OK) {
                 free_graph(g);

@@ -581,37 +581,24 @@ __global__ void __launch_bounds__(1024) cc_list_kernel(GraphArgs g, const int* _
     }
 }
 
-// Members per SM of the cut-local kernel, its threads per member and its list region: as many members as
-// shared memory holds with lists of n / 2 entries, sharing the SM's 2048 threads, but no more than the
-// population spreads over the SMs, and no more than 256 (512) threads up to 1024 (2048) nodes.  Measured at
-// n = 20000 (1023 members of 1000 genes, random generation / hub-heavy fitness, whole call): three of 672
-// threads 68 / 85 us, three of 512 66 / 93; four of 512 hold lists of n / 3 entries only, and hub-heavy members
-// outgrow them.  80 members at n = 5009: 25 us with 1024 threads, 33 with 512.
-struct LocalShape {
-    int per_sm, threads, list_bytes;
-};
+gapa_dev::LocalShape local_shape(const gapa_ctx* c, int s) {
+    return gapa_dev::local_shape(c->g.n, c->g.mean_deg_x16, s,
+                                 gapa_dev::LocalLimits{c->num_sms, c->smem_per_sm, c->smem_reserved, c->fit_smem_max});
+}
 
-LocalShape local_shape(const gapa_ctx* c, int s) {
-    const int n = c->g.n;
-    const size_t bm = gapa_dev::tree16l_bitmap_bytes(n), fixed = gapa_dev::tree16l_smem_bytes(n, 0);
-    const size_t least = std::max(gapa_dev::tree16l_min_list_bytes(n, c->g.mean_deg_x16), bm + (((size_t)n + 15) & ~(size_t)15));
-    const size_t most = bm + (((size_t)n * 2 + 1024 + 15) & ~(size_t)15);
-    int m = std::max(1, std::min(8, (s + c->num_sms - 1) / c->num_sms));
-    for (;; --m) {
-        const size_t block = c->smem_per_sm / (size_t)m, other = c->smem_reserved + 1024;
-        const size_t room = std::min(block > other ? block - other : 0, c->fit_smem_max);
-        if (m == 1 || room >= fixed + least) {
-            const size_t list = std::min(std::max(least, most), (room - fixed) & ~(size_t)15);
-            return LocalShape{m, std::min(n <= 1024 ? 256 : n <= 2048 ? 512 : 1024, (2048 / m) & ~31), (int)list};
-        }
-    }
+// The kernel's fallbacks write as far as the least list region goes: no launch with less.
+int check_shape(const gapa_ctx* c, const gapa_dev::LocalShape& shape) {
+    if ((size_t)shape.list_bytes >= gapa_dev::tree16l_min_list_bytes(c->g.n, c->g.mean_deg_x16)) return GAPA_OK;
+    return gapa_fail(GAPA_ERR_STATE, "cut-local list region of %d bytes for %d nodes", shape.list_bytes, c->g.n);
 }
 
 // The cut-local kernel: members costliest first where not all of them run at once (estimates precomputed by
 // the operator kernel, or here; in order, the calls above take 70 and 97 us).
 int launch_local(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, int k, long long* f, cudaStream_t st,
                  int* kernels, const unsigned* est_in) {
-    const LocalShape shape = local_shape(c, s);
+    const gapa_dev::LocalShape shape = local_shape(c, s);
+    const int rc = check_shape(c, shape);
+    if (rc != GAPA_OK) return rc;
     const int* order = nullptr;
     if (s > shape.per_sm * c->num_sms && s <= kOrderCap) {
         unsigned* e1 = gapa_estimate_buffer(c);
@@ -713,7 +700,9 @@ int launch_piece(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, in
     const size_t parents = gapa_dev::piece_parents_bytes(n);
     const size_t avail = c->piece_smem_max > parents ? c->piece_smem_max - parents : 0;
     const gapa_dev::PieceLayout L = gapa_dev::piece_layout(n, k, kPieceThreads, avail / kPieceTeams);
-    const LocalShape shape = local_shape(c, s);
+    const gapa_dev::LocalShape shape = local_shape(c, s);
+    const int rc = check_shape(c, shape);
+    if (rc != GAPA_OK) return rc;
     if (L.pcap < 512 || s < 2 || s > kOrderCap) return launch_local(c, ga, pop, s, k, f, st, kernels, nullptr);
     unsigned* e1 = gapa_estimate_buffer(c);
     unsigned* e2 = e1 + kOrderCap;

@@ -12,6 +12,7 @@
 #pragma once
 
 #include "gapa_internal.cuh"
+#include "local_layout.cuh"
 
 namespace gapa_dev {
 
@@ -182,14 +183,6 @@ struct Tree16Graph {
     int list_bytes;           // bytes of the member's list region
     int tops_max;             // more tops than this: the full pipeline on 32-bit labels
 };
-
-__host__ __device__ __forceinline__ size_t tree16_lab_bytes(int n) { return ((size_t)n * 2 + 15) & ~(size_t)15; }
-
-// Shared-memory bytes of one member of the full pipeline on 32-bit labels: labels + deleted-node bitmap
-// (reused as a node list once the labels are set) + four team-wide scalars.
-__host__ __device__ __forceinline__ size_t tree32_smem_bytes(int n) {
-    return (size_t)n * 4 + (size_t)((n + 31) >> 5) * 4 + 16;
-}
 
 // The label pick of live node v: its tree parent if live, else its first
 // live lower-numbered neighbour, else v; -1 for a deleted v.
@@ -757,28 +750,6 @@ __device__ __forceinline__ int tree16l_owner(const int* off, int owners, int i) 
 
 constexpr int kLocalLevels = 256;
 constexpr long long kLocalSpinLimit = 1ll << 24;
-
-// Layout of one member: labels (16-byte units for the bulk copy), the list
-// region (16-bit node ids, then the bitmap of listed nodes), twelve team
-// scalars and the mbarrier.
-__host__ __device__ __forceinline__ size_t tree16l_bitmap_bytes(int n) {
-    return ((((size_t)n + 31) >> 5) * 4 + 15) & ~(size_t)15;
-}
-// The tops beyond which a member runs the full pipeline on 32-bit labels, by 16 times the mean degree.
-__host__ __device__ __forceinline__ bool tree16l_sparse(int mean_deg_x16) { return mean_deg_x16 < 80; }
-__host__ __device__ __forceinline__ int tree16l_tops_max(int n, int mean_deg_x16) {
-    return tree16l_sparse(mean_deg_x16) ? n / 8 : n;
-}
-// The least list region: the full pipeline's bitmap and scalars, and 512 entries (sparse graphs: all of
-// the full pipeline on 32-bit labels).
-__host__ __device__ __forceinline__ size_t tree16l_min_list_bytes(int n, int mean_deg_x16) {
-    const size_t least = tree16l_bitmap_bytes(n) + 1024 + 16;
-    const size_t full = tree16l_sparse(mean_deg_x16) ? ((tree32_smem_bytes(n) + 15) & ~(size_t)15) - tree16_lab_bytes(n) : 0;
-    return least > full ? least : full;
-}
-__host__ __device__ __forceinline__ size_t tree16l_smem_bytes(int n, size_t list_bytes) {
-    return tree16_lab_bytes(n) + list_bytes + 48 + 16;
-}
 
 __device__ __forceinline__ unsigned tree16l_smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
