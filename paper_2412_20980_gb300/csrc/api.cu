@@ -63,7 +63,7 @@ void free_graph(DeviceGraph& g) {
     cudaFree(g.sb_line);
     cudaFree(g.sb_col);
     for (SparseForest& f : g.spf) {
-        void* tabs[] = {f.kids, f.croot, f.csize, f.sub, f.bysize, f.cost};
+        void* tabs[] = {f.kids, f.comp, f.csize, f.sub, f.bysize, f.cost};
         for (void* q : tabs) cudaFree(q);
         if (f.owns) {
             void* own[] = {f.perm, f.tparent, f.palt, f.lo_ptr, f.lo_col, f.fptr, f.fcol32, f.fcol16};
@@ -740,6 +740,7 @@ void gapa_destroy(gapa_ctx* c) {
     cudaFree(c->labels);
     cudaFree(c->ig_aux);
     gapa_sparse_release(c);
+    cudaFree(c->sp_head);
     cudaFree(c->sp_order);
     cudaFree(c->sdst_buf);
     for (auto p : c->stage_pop) cudaFree(p);
@@ -768,9 +769,9 @@ int gapa_set_stream(gapa_ctx* c, void* s) {
 }
 
 // A forest of the sparse fitness kernel from a BFS forest of G (or of G without some hubs' edges):
-// children as (first, count) (BFS numbers them consecutively), the root of every node's tree (in BFS
-// order every component is one tree; -1 for single-node components), component sizes at their
-// roots, subtree sizes, the roots by decreasing size (ties: lower root), the per-member cost table
+// children as (first, count) (BFS numbers them consecutively), the components (in BFS order every one
+// is one tree) numbered by decreasing size (ties: lower root): every node's number (-1 for
+// single-node components), their sizes and tree roots; subtree sizes, the per-member cost table
 // by original id (children + 1) and the sum over components of C(size, 2).  With `own`, also the
 // forest's numbering, parents, parent pairs and lower-neighbour and full adjacency in its
 // numbering (rp, col: the graph it was built from).  Returns 1 (nothing uploaded) if some node's
@@ -796,8 +797,14 @@ int upload_sparse_forest(const BfsForest& bf, const std::vector<int32_t>& rp, co
     for (int32_t x = n - 1; x >= 0; --x)
         if (bf.tparent[x] != x) sub[bf.tparent[x]] += sub[x];
     std::stable_sort(roots.begin(), roots.end(), [&](int32_t a, int32_t b) { return csize[a] > csize[b]; });
-    for (int32_t x = 0; x < n; ++x)
-        if (csize[croot[x]] == 1) croot[x] = -1;  // a single-node component: nothing to recount
+    // components numbered by decreasing size; a single-node one has nothing to recount
+    std::vector<int32_t> sizes(roots.size()), number((size_t)n, -1), comp((size_t)n);
+    int multi = 0;
+    for (size_t i = 0; i < roots.size(); ++i) {
+        sizes[i] = csize[roots[i]];
+        if (sizes[i] > 1) number[roots[i]] = multi++;
+    }
+    for (int32_t x = 0; x < n; ++x) comp[x] = number[croot[x]];
     std::vector<int32_t> cost((size_t)n);  // by original id: children + 1
     for (int32_t v = 0; v < n; ++v) cost[v] = kids[bf.perm[v]].y + 1;
     long long pc0 = 0;
@@ -807,7 +814,7 @@ int upload_sparse_forest(const BfsForest& bf, const std::vector<int32_t>& rp, co
                (bytes == 0 || cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess);
     };
     bool ok = up((void**)&f.kids, kids.data(), sizeof(int2) * (size_t)n) &&
-              up((void**)&f.croot, croot.data(), 4 * (size_t)n) && up((void**)&f.csize, csize.data(), 4 * (size_t)n) &&
+              up((void**)&f.comp, comp.data(), 4 * (size_t)n) && up((void**)&f.csize, sizes.data(), 4 * sizes.size()) &&
               up((void**)&f.sub, sub.data(), 4 * (size_t)n) && up((void**)&f.bysize, roots.data(), 4 * roots.size()) &&
               up((void**)&f.cost, cost.data(), 4 * (size_t)n);
     if (ok && own) {
@@ -842,6 +849,7 @@ int upload_sparse_forest(const BfsForest& bf, const std::vector<int32_t>& rp, co
         return gapa_fail(GAPA_ERR_OOM, "sparse fitness forest of %d nodes", n);
     }
     f.ncomp = (int)roots.size();
+    f.multi = multi;
     f.giant = roots.empty() ? -1 : roots[0];
     f.pc0 = pc0;
     return GAPA_OK;
@@ -1122,6 +1130,7 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
         }
     }
     c->g = g;
+    c->sp_refused = gapa_dev::kSpShapes;  // room may have come back
     return GAPA_OK;
 }
 

@@ -34,7 +34,8 @@
 // node of the graph.  One CTA per member at a time, persistent over a work
 // queue; its per-node state (hops, classes, counts, per-component sums) lives
 // in the CTA's own slice of global scratch, which it clears after every
-// member (entries start as -1 / 0 when the scratch is allocated).
+// member (entries start as -1 / 0 when the scratch is allocated; counts are
+// set where a member first touches them).
 #include <climits>
 
 #include "gapa_internal.cuh"
@@ -43,7 +44,11 @@
 namespace {
 
 using gapa_dev::bm_test;
+using gapa_dev::kSpTeams;
+using gapa_dev::kSpThreads;
 using gapa_dev::objective_add;
+using gapa_dev::sp_bitmap_bytes;
+using gapa_dev::sp_smem_bytes;
 using gapa_dev::Team;
 using gapa_dev::team_sum_ll;
 using gapa_dev::tree16l_owner;
@@ -66,12 +71,12 @@ struct SpGraph {
     const int* fptr;      // full adjacency in BFS numbers (CSR)
     const Col* fcol;
     const int2* kids;     // (first child, number of children)
-    const int* croot;     // root of the node's component tree (-1: a single-node component)
-    const int* csize;     // size of the component, at its root
+    const int* comp;      // the node's component by decreasing size (-1: a single-node component)
+    const int* csize;     // size of every component
     const int* sub;       // subtree size
-    const int* bysize;    // component roots by decreasing size (MCN)
+    const int* bysize;    // tree root of every component
     int ncomp;
-    int giant;            // root of the largest component
+    int giant;            // root of the largest component, number 0
     long long pc0;        // sum over components of C(size, 2)
     int objective;        // 0: PC, 1: MCN
 };
@@ -83,30 +88,26 @@ struct SpGraphs {
     SpGraph<Col> f[kSpForests];
 };
 
-// One CTA's slice of the scratch (n entries each).  Reads go through L2 only
-// (__ldcg; a slice moves between SMs from one launch to the next, and within
-// a phase the union-find entries change under other threads' atomics); what a
-// phase writes, later phases read after a barrier.
+// One CTA's slice of the scratch (an entry per node; cl, cacc and best one per component of two nodes or
+// more); as a kernel argument the first CTA's.  Reads go through L2
+// only (__ldcg; a slice moves between SMs from one launch to the next, and
+// within a phase the union-find entries change under other threads' atomics);
+// what a phase writes, later phases read after a barrier.
 struct SpSlot {
     int* hop;                  // live tops: hop, then terminal; -1 elsewhere
     int* cls;                  // terminals: class link (terminal + 1; 0 = R); listed nodes: their class; -1 elsewhere
-    unsigned* cnt;             // terminals: chained subtree weight, then class size; 0 elsewhere
+    unsigned long long* cacc;  // components: deleted << 32 | nodes apart from R; 0 elsewhere
+    unsigned long long* best;  // components whose root is deleted: weight << 32 | ~terminal; 0 elsewhere
+    unsigned* cnt;             // tops that re-picked nothing: chained subtree weight, then class size
     int* list;                 // listed nodes
     int* tl;                   // live tops
     int* th;                   // hop of the live top at the same position of tl (then its terminal)
-    int* cl;                   // touched components (roots), single-node components excepted
-    unsigned long long* cacc;  // component roots: deleted << 32 | nodes apart from R; 0 elsewhere
-    unsigned long long* best;  // component roots whose root is deleted: weight << 32 | ~terminal
+    int* cl;                   // touched components, single-node components excepted
 };
 
 __device__ __forceinline__ int ldcg(const int* p) { return __ldcg(p); }
 __device__ __forceinline__ unsigned ldcg(const unsigned* p) { return __ldcg(p); }
 __device__ __forceinline__ unsigned long long ldcg(const unsigned long long* p) { return __ldcg(p); }
-
-__host__ __device__ __forceinline__ size_t sp_bitmap_bytes(int n) { return ((((size_t)n + 31) >> 5) * 4 + 15) & ~(size_t)15; }
-__host__ __device__ __forceinline__ size_t sp_smem_bytes(int n, int k, int threads) {
-    return sp_bitmap_bytes(n) + (((size_t)2 * k + 1) * 4 + 15) / 16 * 16 + (size_t)3 * threads * 4;
-}
 
 // Class of value a (terminal + 1; 0 = R): the root's value r, with the links
 // on the way that still lie below r pointed at it.  Links always point to
@@ -158,6 +159,12 @@ __device__ __forceinline__ int sp_append(bool want, int v, int lane, int* count,
     const int at = first + __popc(m & ((1u << lane) - 1));
     if (want) list[at] = v;
     return want ? at : -1;
+}
+
+// Tree root of component c.
+template <typename Col>
+__device__ __forceinline__ int sp_root(const SpGraph<Col>& g, int c) {
+    return c == 0 ? g.giant : __ldg(&g.bysize[c]);
 }
 
 // The terminal of live node w's piece: walk up to the first top (its terminal) or tree root.
@@ -267,7 +274,8 @@ __global__ void __launch_bounds__(1024) sp_order_kernel(const unsigned* __restri
 
 template <typename Col, bool SMALL>
 __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_sparse_kernel(const __grid_constant__ SpGraphs<Col> gs, SpSlot base,
-                                                               size_t stride, const int* __restrict__ pop, int s,
+                                                               size_t stride, size_t comps,
+                                                               const int* __restrict__ pop, int s,
                                                                int k, long long* __restrict__ fit, int* head,
                                                                int* status, const int* __restrict__ order, int either) {
     if (either && (head[1] != 0) != SMALL) return;  // the other shape's launch takes the call
@@ -284,16 +292,16 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
     int* s_first = s_off + T;
     int* s_val = s_first + T;
     int* ws = reinterpret_cast<int*>(red);
-    const size_t o = (size_t)blockIdx.x * stride;
+    const size_t o = (size_t)blockIdx.x * stride, oc = (size_t)blockIdx.x * comps;
     int* const hop = base.hop + o;
     int* const cls = base.cls + o;
     unsigned* const cnt = base.cnt + o;
     int* const list = base.list + o;
     int* const tl = base.tl + o;
     int* const th = base.th + o;
-    int* const cl = base.cl + o;
-    unsigned long long* const cacc = base.cacc + o;
-    unsigned long long* const best = base.best + o;
+    int* const cl = base.cl + oc;
+    unsigned long long* const cacc = base.cacc + oc;
+    unsigned long long* const best = base.best + oc;
     constexpr int F = kSpInFlight;
 
     for (;;) {
@@ -362,8 +370,8 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
             int gdel = 0;  // deletions in the largest component, summed in shared memory
             for (int i0 = tid & ~31; i0 < nd; i0 += T) {
                 const int i = i0 + lane;
-                int c = i < nd ? __ldg(&g.croot[D[i]]) : -1;  // -1: a single-node component
-                if (c >= 0 && c == g.giant) {
+                int c = i < nd ? __ldg(&g.comp[D[i]]) : -1;  // -1: a single-node component
+                if (c == 0) {
                     ++gdel;
                     c = -1;
                 }
@@ -372,7 +380,8 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
                     const unsigned long long old = atomicAdd(&cacc[c], (unsigned long long)__popc(peers) << 32);
                     if (old == 0ull) {
                         cl[atomicAdd(&s_ncl, 1)] = c;
-                        if (!bm_test(dead, c)) cls[c] = c + 1;  // a live tree root is a terminal
+                        const int root = sp_root(g, c);
+                        if (!bm_test(dead, root)) cls[root] = root + 1;  // a live tree root is a terminal
                     }
                 }
             }
@@ -381,10 +390,9 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
         }
         tm.sync();
         if (tid == 0 && s_gdel) {
-            const int c = g.giant;
-            cacc[c] = (unsigned long long)s_gdel << 32;
-            cl[s_ncl++] = c;
-            if (!bm_test(dead, c)) cls[c] = c + 1;
+            cacc[0] = (unsigned long long)s_gdel << 32;
+            cl[s_ncl++] = 0;
+            if (!bm_test(dead, g.giant)) cls[g.giant] = g.giant + 1;
         }
 
         // 2. re-pick and hop of every top; the live tops are also listed compactly (tl) for the
@@ -437,6 +445,7 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
                     }
                 }
                 hop[t[u]] = x;
+                if (x == t[u]) cnt[x] = 0u;
                 y[u] = x;
             }
 #pragma unroll
@@ -495,8 +504,8 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
                 }
                 if (t[u] >= 0) {
                     // x is a top that re-picked nothing, or a live tree root (never weighed)
-                    const int cx = __ldg(&g.croot[x[u]]);
-                    if (cx >= 0 && bm_test(dead, cx)) {
+                    const int cx = __ldg(&g.comp[x[u]]);
+                    if (cx >= 0 && bm_test(dead, sp_root(g, cx))) {
                         key = x[u];
                         wgt = (unsigned)__ldg(&g.sub[t[u]]);
                     }
@@ -539,8 +548,8 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
         // 3. reference terminal of components whose root is deleted
         for (int j = tid; j < nterm; j += T) {
             const int t = ldcg(&list[j]);
-            const int c = __ldg(&g.croot[t]);
-            if (bm_test(dead, c))
+            const int c = __ldg(&g.comp[t]);
+            if (bm_test(dead, sp_root(g, c)))
                 atomicMax(&best[c], ((unsigned long long)ldcg(&cnt[t]) << 32) | (unsigned long long)(~(unsigned)t));
         }
         tm.sync();
@@ -548,9 +557,10 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
         const int ncl = s_ncl;
         for (int i = tid; i < ncl; i += T) {
             const int c = ldcg(&cl[i]);
+            const int root = sp_root(g, c);
             int r;
-            if (!bm_test(dead, c)) {
-                r = c + 1;
+            if (!bm_test(dead, root)) {
+                r = root + 1;
             } else {
                 const unsigned long long bk = ldcg(&best[c]);
                 if (bk == 0ull) continue;  // no live node left in the component
@@ -567,8 +577,8 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
         // every terminal's and live root's link straight to its class root (0: R)
         for (int j = tid; j < nterm; j += T) sp_find(cls, ldcg(&list[j]) + 1);
         for (int i = tid; i < ncl; i += T) {
-            const int c = ldcg(&cl[i]);
-            if (!bm_test(dead, c)) sp_find(cls, c + 1);
+            const int root = sp_root(g, ldcg(&cl[i]));
+            if (!bm_test(dead, root)) sp_find(cls, root + 1);
         }
         tm.sync();
 
@@ -676,7 +686,7 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
             if (i < nl) {
                 const int v = ldcg(&list[i]);
                 r = sp_find(cls, ldcg(&cls[v]));
-                if (r != 0) c = __ldg(&g.croot[v]);
+                if (r != 0) c = __ldg(&g.comp[v]);
             }
             const unsigned pr = __match_any_sync(0xffffffffu, r);
             if (r != 0 && lane == __ffs(pr) - 1) atomicAdd(&cnt[r - 1], (unsigned)__popc(pr));
@@ -703,10 +713,10 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
             if (mx) {
                 // the largest untouched component
                 for (int j = 0; j < g.ncomp; ++j) {
-                    const int c = __ldg(&g.bysize[j]);
-                    const bool touched = __ldg(&g.csize[c]) == 1 ? bm_test(dead, c) : ldcg(&cacc[c]) != 0ull;
-                    if (!touched) {
-                        const long long cs = __ldg(&g.csize[c]);
+                    // a deleted root touches its component; a live one of a touched component holds a class link
+                    const int root = __ldg(&g.bysize[j]);
+                    if (!bm_test(dead, root) && ldcg(&cls[root]) == -1) {
+                        const long long cs = __ldg(&g.csize[j]);
                         tot = cs > tot ? cs : tot;
                         break;
                     }
@@ -736,16 +746,13 @@ __global__ void __launch_bounds__(SMALL ? 512 : kSpBlock, SMALL ? 3 : 1) cc_spar
             for (int u = 0; u < F; ++u) v[u] = i0 + u * T < nl ? ldcg(&list[i0 + u * T]) : -1;
 #pragma unroll
             for (int u = 0; u < F; ++u)
-                if (v[u] >= 0) {
-                    cls[v[u]] = -1;
-                    cnt[v[u]] = 0u;
-                }
+                if (v[u] >= 0) cls[v[u]] = -1;
         }
         for (int i = tid; i < ncl; i += T) {
             const int c = ldcg(&cl[i]);
             cacc[c] = 0ull;
             best[c] = 0ull;
-            cls[c] = -1;
+            cls[sp_root(g, c)] = -1;
         }
         tm.sync();
     }
@@ -763,7 +770,7 @@ SpGraph<Col> sp_graph(const gapa_ctx* c, const SparseForest& f, const Col* fcol)
     g.fptr = f.fptr;
     g.fcol = fcol;
     g.kids = f.kids;
-    g.croot = f.croot;
+    g.comp = f.comp;
     g.csize = f.csize;
     g.sub = f.sub;
     g.bysize = f.bysize;
@@ -791,26 +798,8 @@ bool gapa_sparse_fits(const gapa_ctx* c, int k) {
     return c->g.sp_nforests > 0 && c->sp_smem_max > 0 && sp_smem_bytes(c->g.n, k, kSpBlock) <= c->sp_smem_max;
 }
 
-// Teams per SM and their threads: 1 x 1024, 2 x 512, 4 or 6 x 256 (the small teams' kernel is held to 42
-// registers), the most that leave every SM two rounds of members to balance, that shared memory holds and
-// that keep the scratch within 4 GB.  A member's phases wait at barriers and on scattered reads, so several
-// smaller teams cover each other; with a single round the largest member, now on fewer threads, is what the
-// call waits for (310 members of 2000 genes, n = 70000, BA(3): 139 us at 1 per SM, 167 at 2).  At 1 / 2 / 4
-// per SM: 620 members 227 / 183 / 283 us, 1300 members 416 / 300 / 294.  One (mu+lambda) generation with 2048
-// children (2000 genes, n = 100000, BA(3)), at 1 / 2 / 4 / 6: 706 / 529 / 510 / 472 us.  Members of uneven cost
-// (up to all genes among the hubs, n = 100000) go the other way, 2048 of them 3551 / 3620 / 4396 / 3872, 762 of
-// them 1421 / 1734 at 1 / 2: the order kernel keeps such calls at one member per SM.
-constexpr int kSpTeams[4] = {1, 2, 4, 6}, kSpThreads[4] = {1024, 512, 256, 256};
-
 static int sp_shape(const gapa_ctx* c, int s, int k) {
-    int i = 3;
-    for (; i > 0; --i) {
-        const long long teams = (long long)kSpTeams[i] * c->num_sms;
-        if (s >= 2 * teams && (size_t)teams * c->g.n * 44 <= ((size_t)4 << 30) &&
-            kSpTeams[i] * (sp_smem_bytes(c->g.n, k, kSpThreads[i]) + c->smem_reserved + 1024) <= c->smem_per_sm)
-            break;
-    }
-    return i;
+    return gapa_dev::sp_shape(c->g.n, s, k, gapa_dev::SpLimits{c->num_sms, c->smem_per_sm, c->smem_reserved});
 }
 
 int gapa_sparse_init(gapa_ctx* c) {
@@ -826,79 +815,88 @@ int gapa_sparse_init(gapa_ctx* c) {
 }
 
 void gapa_sparse_release(gapa_ctx* c) {
-    cudaFree(c->sp_scratch);
-    c->sp_scratch = nullptr;
-    c->sp_scratch_cap = 0;
-    for (void*& old : c->sp_old) {
-        cudaFree(old);
-        old = nullptr;
+    for (void*& block : c->sp_block) {
+        cudaFree(block);
+        block = nullptr;
     }
+    c->sp_held = -1;
 }
 
-// Scratch of the persistent CTAs: nine n-entry arrays per CTA (hops, classes,
-// counts, listed nodes, live tops, their hops, touched components: int32;
-// per-component sums and reference keys: int64).  All but the lists are set to
-// -1 / 0 once here and left that way by every member.  A larger population may ask for more slices: the
-// smaller block then stays until the context or the graph goes, as captured work
-// may still point to it.
-int gapa_sparse_prepare(gapa_ctx* c, int s) {
-    const int n = c->g.n;
-    const size_t stride = ((size_t)n + 63) & ~(size_t)63;
-    // member order, estimates and forests (3 ints per member)
+// A block of slices for `shape`, each array holding all of them after one another; hops and classes at -1,
+// component sums at 0.
+static bool sp_new_block(gapa_ctx* c, int shape) {
+    const size_t slots = (size_t)c->num_sms * kSpTeams[shape];
+    void* p = nullptr;
+    if (cudaMalloc(&p, slots * gapa_dev::sp_slice_bytes(c->sp_stride, c->sp_comps)) != cudaSuccess ||
+        cudaMemsetAsync(p, 0xFF, slots * c->sp_stride * 8) != cudaSuccess ||
+        cudaMemsetAsync(static_cast<char*>(p) + slots * c->sp_stride * 24, 0, slots * c->sp_comps * 20) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(p);
+        return false;
+    }
+    c->sp_block[shape] = p;
+    return true;
+}
+
+// Whether a stream is being captured: no scratch is allocated then.
+static bool sp_captured(cudaStream_t st) {
+    cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &state) == cudaSuccess) return state != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// Scratch for s members: the member order, estimates and forests (3 ints per member), and the block of the
+// call's shape, or of the next smaller one that the device has room for (a population of 2048 at n = 100000
+// takes six slices of 2.4 MB per SM, 2.2 GB).  A smaller block stays beside a larger one, as captured work may
+// point to it, until the context goes or a graph comes that has another number of nodes or more components.
+int gapa_sparse_prepare(gapa_ctx* c, int s, cudaStream_t st) {
+    const size_t stride = ((size_t)c->g.n + 63) & ~(size_t)63;
     if ((size_t)3 * std::max(s, 1) > c->sp_order_cap) {
         int rc = gapa_reserve((void**)&c->sp_order, &c->sp_order_cap, (size_t)3 * std::max(s, 1), sizeof(int));
         if (rc != GAPA_OK) return rc;
     }
-    const int slots = c->num_sms * kSpTeams[sp_shape(c, s, 0)];
-    if (c->sp_scratch && c->sp_stride == stride && c->sp_slots >= slots) return GAPA_OK;  // (also inside a stream capture)
-    const size_t bytes = (size_t)slots * stride * (7 * 4 + 2 * 8) + 64;
-    if (c->sp_stride != stride) gapa_sparse_release(c);
-    void* block = nullptr;
-    if (cudaMalloc(&block, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        if (c->sp_scratch) return GAPA_OK;  // the smaller block serves
-        return gapa_fail(GAPA_ERR_OOM, "sparse fitness scratch of %zu bytes", bytes);
+    if (!c->sp_head) GAPA_CUDA(cudaMalloc(&c->sp_head, 2 * sizeof(int)));
+    size_t comps = 0;
+    for (const SparseForest& f : c->g.spf) comps = std::max(comps, ((size_t)f.multi + 15) & ~(size_t)15);
+    if (c->sp_stride != stride || c->sp_comps < comps) {
+        gapa_sparse_release(c);
+        c->sp_stride = stride;
+        c->sp_comps = comps;
     }
-    for (void*& old : c->sp_old)
-        if (!old) {
-            old = c->sp_scratch;
-            break;
-        }
-    c->sp_scratch = block;
-    c->sp_scratch_cap = bytes;
-    c->sp_stride = stride;
-    c->sp_slots = slots;
-    const size_t ints = (size_t)slots * stride;
-    char* p = static_cast<char*>(c->sp_scratch);
-    // hop, cls = -1; cnt, cacc, best = 0 (the lists are read only as far as a member wrote them); the queue head last
-    GAPA_CUDA(cudaMemsetAsync(p, 0xFF, ints * 8));
-    GAPA_CUDA(cudaMemsetAsync(p + ints * 8, 0, ints * 4));
-    GAPA_CUDA(cudaMemsetAsync(p + ints * 28, 0, ints * 16 + 64));
-    GAPA_CUDA(cudaDeviceSynchronize());
+    const int shape = sp_shape(c, s, 0);
+    if (shape <= c->sp_held || (c->sp_held >= 0 && c->sp_held + 1 >= c->sp_refused)) return GAPA_OK;
+    const int before = c->sp_held;
+    const bool captured = c->capturing || sp_captured(st);
+    c->sp_held = gapa_dev::sp_grow(before, shape, !captured, &c->sp_refused, [&](int i) { return sp_new_block(c, i); });
+    if (c->sp_held < 0)
+        return gapa_fail(GAPA_ERR_OOM, "sparse fitness scratch of %zu bytes",
+                         gapa_dev::sp_slice_bytes(stride, c->sp_comps) * (size_t)c->num_sms);
+    if (c->sp_held > before) GAPA_CUDA(cudaDeviceSynchronize());
     return GAPA_OK;
 }
 
 int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
                                int* kernels) {
     if (!gapa_sparse_fits(c, k)) return gapa_fail(GAPA_ERR_INVALID_ARG, "sparse fitness: shared memory too small");
-    int rc = gapa_sparse_prepare(c, s);
+    int rc = gapa_sparse_prepare(c, s, st);
     if (rc != GAPA_OK) return rc;
-    const size_t ints = (size_t)c->sp_slots * c->sp_stride;
-    char* p = static_cast<char*>(c->sp_scratch);
+    // the arrays of the largest block, whatever shape runs
+    const size_t slots = (size_t)c->num_sms * kSpTeams[c->sp_held], nodes = slots * c->sp_stride, comps = slots * c->sp_comps;
+    int* const node = static_cast<int*>(c->sp_block[c->sp_held]);
     SpSlot b;
-    b.hop = reinterpret_cast<int*>(p);
-    b.cls = reinterpret_cast<int*>(p + ints * 4);
-    b.cnt = reinterpret_cast<unsigned*>(p + ints * 8);
-    b.list = reinterpret_cast<int*>(p + ints * 12);
-    b.tl = reinterpret_cast<int*>(p + ints * 16);
-    b.th = reinterpret_cast<int*>(p + ints * 20);
-    b.cl = reinterpret_cast<int*>(p + ints * 24);
-    b.cacc = reinterpret_cast<unsigned long long*>(p + ints * 28);
-    b.best = reinterpret_cast<unsigned long long*>(p + ints * 36);
-    int* head = reinterpret_cast<int*>(p + ints * 44);
+    b.hop = node;
+    b.cls = node + nodes;
+    b.cnt = reinterpret_cast<unsigned*>(node + 2 * nodes);
+    b.list = node + 3 * nodes;
+    b.tl = node + 4 * nodes;
+    b.th = node + 5 * nodes;
+    b.cl = node + 6 * nodes;
+    b.cacc = reinterpret_cast<unsigned long long*>(b.cl + comps);
+    b.best = b.cacc + comps;
+    int* head = c->sp_head;  // queue head, then the order kernel's choice of shape
     GAPA_CUDA(cudaMemsetAsync(head, 0, sizeof(int), st));
-    int shape = sp_shape(c, s, k);
-    while (shape > 0 && c->num_sms * kSpTeams[shape] > c->sp_slots) --shape;  // (a smaller block had to serve)
+    const int shape = std::min(sp_shape(c, s, k), c->sp_held);  // (a smaller block may have to serve)
     // every member's forest and cost estimate, then the members costliest first
     unsigned* est = reinterpret_cast<unsigned*>(c->sp_order + s);
     int* forest = c->sp_order + 2 * (size_t)s;
@@ -912,7 +910,7 @@ int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, in
     // a call that may run in small teams launches both shapes, one of which returns at once (about 3 us)
     auto launch = [&](auto kernel, auto graphs, int i) {
         const int T = kSpThreads[i], grid = std::min(c->num_sms * kSpTeams[i], std::max(s, 1));
-        kernel<<<grid, T, sp_smem_bytes(c->g.n, k, T), st>>>(graphs, b, c->sp_stride, pop, s, k,
+        kernel<<<grid, T, sp_smem_bytes(c->g.n, k, T), st>>>(graphs, b, c->sp_stride, c->sp_comps, pop, s, k,
                                                             reinterpret_cast<long long*>(fit), head, c->status,
                                                             c->sp_order, shape > 0);
     };

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/gapa.h"
+#include "sparse_layout.cuh"
 
 // ---------------------------------------------------------------------------
 // Device status word: kernels OR these bits in; gapa_sync() reports them.
@@ -117,10 +118,10 @@ struct DeviceForest {
 
 // One BFS forest of the sparse fitness kernel (fitness_sparse.cu): numbering, tree parents, the
 // (tree parent, second lower neighbour) pairs, lower-neighbour and full adjacency CSR in its
-// numbering, and per node (first child, children), the root of its component tree (-1 for a
-// single-node component), the component's size at its root, subtree sizes, the component roots by
-// decreasing size, and by original id the member cost estimate (children + 1); the number of
-// components, the largest one's root and the sum over components of C(size, 2).  `owns`: the
+// numbering, and per node (first child, children), its component (numbered by decreasing size, -1
+// for a single-node one) and subtree size, per component its size and tree root, and by original id
+// the member cost estimate (children + 1); the number of components and of those of two nodes or
+// more, the largest one's root and the sum over components of C(size, 2).  `owns`: the
 // numbering and adjacency arrays are this forest's own (forest 0 borrows the graph's).
 struct SparseForest {
     int* perm = nullptr;
@@ -132,12 +133,12 @@ struct SparseForest {
     int* fcol32 = nullptr;
     unsigned short* fcol16 = nullptr;
     int2* kids = nullptr;
-    int* croot = nullptr;
+    int* comp = nullptr;
     int* csize = nullptr;
     int* sub = nullptr;
     int* bysize = nullptr;
     int* cost = nullptr;
-    int ncomp = 0;
+    int ncomp = 0, multi = 0;
     int giant = -1;
     long long pc0 = 0;
     bool owns = false;
@@ -242,11 +243,12 @@ struct gapa_ctx {
     int* status = nullptr;  // device status word
     // scratch owned by the context
     int* labels = nullptr;  // global label scratch for graphs too large for shared memory
-    void* sp_scratch = nullptr;  // per-CTA state of the sparse fitness kernel (hops, classes, counts, lists, sums)
-    size_t sp_scratch_cap = 0;   // bytes
-    size_t sp_stride = 0;        // entries per CTA slice
-    int sp_slots = 0;            // CTA slices
-    void* sp_old[3] = {nullptr, nullptr, nullptr};  // smaller blocks that captured work may still use
+    void* sp_block[gapa_dev::kSpShapes] = {};  // slices of the sparse fitness kernel's CTAs, by launch shape
+    int sp_held = -1;            // the largest shape whose block is held
+    int sp_refused = gapa_dev::kSpShapes;  // the smallest shape whose block the device had no room for
+    size_t sp_stride = 0;        // entries per node array of a slice
+    size_t sp_comps = 0;         // and per component array
+    int* sp_head = nullptr;      // queue head and choice of shape
     size_t sp_smem_max = 0;      // max dynamic shared memory of the sparse fitness kernel
     int* sp_order = nullptr;     // the sparse kernel's member order (member | forest << 28), then the
                                  // members' cost estimates and forests
@@ -419,7 +421,7 @@ int gapa_ig_prepare(gapa_ctx* c, int s);
 // context's graph, its one-time set-up, its scratch (outside any capture) and its launch.
 bool gapa_sparse_fits(const gapa_ctx* c, int k);
 int gapa_sparse_init(gapa_ctx* c);
-int gapa_sparse_prepare(gapa_ctx* c, int s);
+int gapa_sparse_prepare(gapa_ctx* c, int s, cudaStream_t st);
 void gapa_sparse_release(gapa_ctx* c);
 int gapa_launch_fitness_sparse(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
                                int* kernels = nullptr);
