@@ -229,8 +229,10 @@ __global__ void __launch_bounds__(1024) sp_cost_kernel(const int* __restrict__ p
 // the persistent CTAs take the costliest members first and none starts late; entry = member |
 // forest << 28.  Where the call may run in small teams, `slots` of them, *small says whether it does:
 // when the costliest member, on its share of an SM, is no more than its slot's share of the sum of
-// the estimates (else that member is what the call waits for; see sp_shape), and the members are light,
-// four tops a gene at the mean (two for random genes; heavier members fill their SM's scattered accesses).
+// the estimates (else that member is what the call waits for; see sp_shape), and the members are light, two and
+// a half a gene at the mean.  The estimate of random genes is one and a half to two; that of hub-heavy sets 2.8 to
+// 76, and these fill their SM's scattered accesses: time against one team per SM 0.68 to 1.65, 0.56 to 2.3 and
+// 0.47 to 1.5 at two, four and six teams.
 __global__ void __launch_bounds__(1024) sp_order_kernel(const unsigned* __restrict__ est,
                                                         const int* __restrict__ forest, int s,
                                                         int* __restrict__ order, int slots, int k, int* __restrict__ small) {
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(1024) sp_order_kernel(const unsigned* __restri
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        *small = (unsigned long long)most * (unsigned)slots <= sum && sum <= 4ull * (unsigned)k * (unsigned)s;
+        *small = (unsigned long long)most * (unsigned)slots <= sum && 2 * sum <= 5ull * (unsigned)k * (unsigned)s;
         int acc = 0;
         for (int c = 0; c < 33; ++c) {
             const int x = cnt[c];
@@ -799,7 +801,7 @@ bool gapa_sparse_fits(const gapa_ctx* c, int k) {
 }
 
 static int sp_shape(const gapa_ctx* c, int s, int k) {
-    return gapa_dev::sp_shape(c->g.n, s, k, gapa_dev::SpLimits{c->num_sms, c->smem_per_sm, c->smem_reserved});
+    return gapa_dev::sp_shape(c->g.n, c->g.mean_deg_x16, s, k, gapa_dev::SpLimits{c->num_sms, c->smem_per_sm, c->smem_reserved});
 }
 
 int gapa_sparse_init(gapa_ctx* c) {

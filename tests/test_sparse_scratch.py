@@ -18,6 +18,7 @@ using namespace gapa_dev;
 extern "C" int grow(int held, int shape, int may_grow, int* refused, int room, int* asked) {
     return sp_grow(held, shape, may_grow != 0, refused, [&](int i) { ++*asked; return i < room; });
 }
+extern "C" int shape(int n, int deg16, int s, int k) { return sp_shape(n, deg16, s, k, SpLimits{152, 228 * 1024, 1024}); }
 """
 
 
@@ -30,10 +31,10 @@ def layout(tmp_path_factory):
     return ctypes.CDLL(str(d / "grow.so"))
 
 
-@pytest.mark.parametrize("room", range(5))
-@pytest.mark.parametrize("held,shape", [(-1, 0), (-1, 3), (0, 3), (0, 2), (2, 1), (2, 3)])
+@pytest.mark.parametrize("room", range(4))
+@pytest.mark.parametrize("held,shape", [(-1, 0), (-1, 2), (0, 2), (0, 1), (2, 1), (1, 2)])
 def test_growth_steps_down_and_asks_once(layout, room, held, shape):
-    refused, asked = ctypes.c_int(4), ctypes.c_int(0)
+    refused, asked = ctypes.c_int(3), ctypes.c_int(0)
     call = lambda h, s, may=1: layout.grow(h, s, may, ctypes.byref(refused), room, ctypes.byref(asked))
     want = max(held, min(shape, room - 1))
     assert call(held, shape) == want  # the largest that there is room for, and none given up
@@ -43,9 +44,41 @@ def test_growth_steps_down_and_asks_once(layout, room, held, shape):
 
 
 def test_no_growth_inside_a_capture(layout):
-    refused, asked = ctypes.c_int(4), ctypes.c_int(0)
-    assert layout.grow(0, 3, 0, ctypes.byref(refused), 4, ctypes.byref(asked)) == 0
-    assert asked.value == 0 and refused.value == 4
+    refused, asked = ctypes.c_int(3), ctypes.c_int(0)
+    assert layout.grow(0, 2, 0, ctypes.byref(refused), 3, ctypes.byref(asked)) == 0
+    assert asked.value == 0 and refused.value == 3
+
+
+# what small teams were measured slower on keeps one member per SM: trees and graphs of mean degree 3, less
+# than eight members per SM, more nodes than the slices' reads stay in L2 for
+@pytest.mark.parametrize("n,deg16,s,k,want", [
+    (60000, 32, 4096, 200, 0), (200000, 48, 4096, 2000, 0), (60000, 56, 1216, 200, 1),
+    (100000, 96, 1215, 2000, 0), (100000, 96, 1216, 2000, 1), (100000, 96, 1823, 2000, 1), (100000, 96, 1824, 2000, 2),
+    (109649, 96, 2048, 2000, 2), (109650, 96, 2048, 2000, 1), (263157, 128, 4096, 2000, 1),
+    (263158, 128, 4096, 2000, 0), (1 << 20, 128, 4096, 200, 0)])
+def test_small_teams_where_they_gain(layout, n, deg16, s, k, want):
+    assert layout.shape(n, deg16, s, k) == want
+
+
+# the shapes that the device chooses between, by the launches of a call (cost, order, and one kernel or both)
+@pytest.mark.gpu
+@pytest.mark.parametrize("graph,per_sm,launches", [("ba", 8, 4), ("ba", 12, 4), ("tree", 12, 3)])
+def test_shapes_on_both_sides_of_a_rule_match_oracle(ctx, graph, per_sm, launches):
+    import torch
+
+    n, sms = 1500, torch.cuda.get_device_properties(0).multi_processor_count
+    g = synth.ba_graph(n, 3 if graph == "ba" else 1, 1)
+    ctx.graph_upload(g.row_ptr, g.col)
+    order = np.argsort(-g.degrees(), kind="stable").astype(np.int32)
+    for s, want in ((per_sm * sms - 1, 3 if per_sm == 8 else launches), (per_sm * sms, launches)):
+        for hubs in (False, True):  # light members alike, heavy ones
+            pop = synth.random_deletion_sets(n, 75, s, s)
+            if hubs:
+                pop[:, :40] = order[:40]
+            ctx.profile_begin()
+            got = _fitness(ctx, pop)
+            assert ctx.profile_end()["fitness_launches"] == want
+            assert np.array_equal(got, oracle.fitness(g.row_ptr, g.col, pop, nthreads=oracle.max_threads())), (s, hubs)
 
 
 @pytest.fixture(scope="module")
@@ -123,7 +156,7 @@ def test_members_and_graphs_leave_nothing_behind(ctx, objective):
                                           synth.named_graph("empty", 100), synth.ba_graph(400, 2, 2))]
     ctx.set_objective(OBJECTIVE_MCN if objective == "mcn" else OBJECTIVE_PC)
     try:
-        for s in (sms, 13 * sms, 3, 6 * sms):
+        for s in (sms, 13 * sms, 3, 8 * sms):
             for g in graphs:
                 ctx.graph_upload(g.row_ptr, g.col)
                 order = np.argsort(-g.degrees(), kind="stable").astype(np.int32)
