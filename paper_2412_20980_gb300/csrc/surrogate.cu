@@ -313,14 +313,19 @@ __global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop
                                                      const int* __restrict__ col, ResidRow* __restrict__ out,
                                                      unsigned long long* __restrict__ sums, double* __restrict__ ms) {
     extern __shared__ unsigned bm[];
-    __shared__ int red[3][32];
-    __shared__ bool s_last;
-    __shared__ int s_list[kOnce ? kResidList : 1], s_count;
-    __shared__ int2 s_own[32][32];  // per warp: of the genes with dealt arcs, first arc less prefix, and the gene
+    __shared__ int red[3][8];  // counts (eight partial sums each), then whether this row is the last
     const int r = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (r >= rows) return;
     const int words = (n + 31) >> 5;
     unsigned *once = bm + words, *twice = once + words;
+    // of a warp's genes with dealt arcs, first arc less prefix, and the gene (without the bitmaps in registers:
+    // the deletion bitmap alone may take all but a few bytes of shared memory)
+    int2* own = nullptr;
+    if constexpr (kOnce) {
+        __shared__ int2 s_own[32][32];
+        own = s_own[warp];
+    }
+    if (t < 24) (&red[0][0])[t] = 0;
     for (int w = t; w < words; w += blockDim.x) {
         bm[w] = 0u;
         if (kOnce) {
@@ -366,17 +371,33 @@ __global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31), start = incl - d;
         const unsigned dealt = __ballot_sync(0xffffffffu, d > 0);
-        __syncwarp();
-        if (d > 0) s_own[warp][__popc(dealt & ((1u << lane) - 1))] = make_int2(b - start, v);
-        __syncwarp();
+        int2 nth = make_int2(0, 0);  // without the bitmaps: the lane-th of those genes
+        if constexpr (kOnce) {
+            __syncwarp();
+            if (d > 0) own[__popc(dealt & ((1u << lane) - 1))] = make_int2(b - start, v);
+            __syncwarp();
+        } else {
+            int at = 0, left = lane;
+#pragma unroll
+            for (int w = 16; w > 0; w >>= 1) {
+                const int c = __popc((dealt >> at) & ((1u << w) - 1));
+                if (left >= c) {
+                    left -= c;
+                    at += w;
+                }
+            }
+            nth = make_int2(__shfl_sync(0xffffffffu, b - start, at & 31), __shfl_sync(0xffffffffu, v, at & 31));
+        }
         int before = 0;  // genes that start in earlier steps
         for (int base = 0; base < total; base += 32) {
             const unsigned at = (unsigned)(start - base);
             const unsigned starts = __reduce_or_sync(0xffffffffu, d > 0 && at < 32u ? 1u << at : 0u);
-            const int idx = base + lane;
-            if (idx < total) {
-                const int2 own = s_own[warp][before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
-                arc(own.y, __ldg(col + own.x + idx));
+            const int idx = base + lane, g = before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+            if constexpr (kOnce) {
+                if (idx < total) arc(own[g].y, __ldg(col + own[g].x + idx));
+            } else {
+                const int x = __shfl_sync(0xffffffffu, nth.x, g & 31), y = __shfl_sync(0xffffffffu, nth.y, g & 31);
+                if (idx < total) arc(y, __ldg(col + x + idx));
             }
             before += __popc(starts);
         }
@@ -389,7 +410,8 @@ __global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop
             for (int p = bb + lane; p < eb; p += 32) arc(vb, __ldg(col + p));
         }
     }
-    if (kOnce) {
+    if constexpr (kOnce) {
+        __shared__ int s_list[kResidList], s_count;
         // a row with repeated genes counts a node once per gene equal to its first deleted neighbour
         auto times = [&](int v) {
             if (!repeated) return 1;
@@ -433,14 +455,14 @@ __global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop
         c2 += __shfl_down_sync(0xffffffffu, c2, o);
     }
     if (lane == 0) {
-        red[0][warp] = c0;
-        red[1][warp] = c1;
-        red[2][warp] = c2;
+        atomicAdd(&red[0][warp & 7], c0);
+        atomicAdd(&red[1][warp & 7], c1);
+        atomicAdd(&red[2][warp & 7], c2);
     }
     __syncthreads();
     if (t == 0) {
         int x = 0, y = 0, z = 0;
-        for (int w = 0; w < nwarps; ++w) {
+        for (int w = 0; w < 8; ++w) {
             x += red[0][w];
             y += red[1][w];
             z += red[2][w];
@@ -453,10 +475,10 @@ __global__ void __launch_bounds__(1024) resid_kernel(const int* __restrict__ pop
             atomicAdd(&sums[3 + j], c[j] * c[j]);
         }
         __threadfence();
-        s_last = atomicAdd(&sums[6], 1ull) == (unsigned long long)rows - 1;
+        red[0][0] = atomicAdd(&sums[6], 1ull) == (unsigned long long)rows - 1;
     }
     __syncthreads();
-    if (!s_last || t >= 7) return;
+    if (!red[0][0] || t >= 7) return;
     __threadfence();
     if (t < 3) {
         const double s1 = (double)(long long)__ldcg(&sums[t]), s2 = (double)(long long)__ldcg(&sums[3 + t]);
