@@ -180,8 +180,8 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(GemmArgs a) {
 // mean degree 6): 143 us.  A gather of the head's entry of the
 // neighbour table per arc took 274 us with two neighbours per entry and 222 us with
 // four (bound by the L1's 32 tag lookups per gather), and stays where three
-// bitmaps exceed shared memory; the bitmaps with a binary search per arc and a
-// list appended to arc by arc 158 us.
+// bitmaps exceed shared memory or cost more than they settle (resid_shape); the
+// bitmaps with a binary search per arc and a list appended to arc by arc 158 us.
 __device__ __forceinline__ bool bm_dead(const unsigned* bm, int w) { return (bm[w >> 5] >> (w & 31)) & 1u; }
 
 // Per node: its four neighbours of lowest degree (earlier arcs first among equals; -1 when absent).  Any
@@ -228,6 +228,8 @@ __device__ __forceinline__ int live_upto2(const unsigned* bm, const int4* __rest
                                           int* first_dead, int* w) {
     const int4 tu = __ldg(T + u);
     const int x[4] = {tu.x, tu.y, tu.z, tu.w == -1 ? -1 : tu.w & INT_MAX};
+    // (most are settled here where the genes are few: without this exit an arc of a hub costs two more tests)
+    if (x[1] >= 0 && !bm_dead(bm, x[0]) && !bm_dead(bm, x[1])) return 2;
     int live = 0, fd = INT_MAX, lw = -1;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1129,6 +1131,8 @@ struct gapa_surrogate {
     size_t resid_smem = 0;       // bytes of one bitmap of resid_kernel
     bool resid_once = false;     // its three bitmaps fit in shared memory
     unsigned* low = nullptr;     // bitmap of the nodes of degree one and two
+    int max_degree = 0;
+    double mean_degree = 0;
     int* batch_rows = nullptr;
     double* stats = nullptr;
     int tau = 0;
@@ -1174,19 +1178,52 @@ int refresh_bf16(gapa_surrogate* s, cudaStream_t st) {
 
 int round16(int x) { return (x + 15) & ~15; }
 
+// Variant of resid_kernel (with the once / twice bitmaps, or the deletion bitmap alone) and threads per row.
+struct ResidShape {
+    bool once;
+    int threads;
+};
+
+// The once / twice bitmaps settle an arc with one shared-memory atomic, but each row clears and reads three
+// bitmaps, and these keep rows off an SM.  They pay where a row has many arcs for its words, where lists are
+// long (a node of degree 128: without the bitmaps 0.76 to 0.96 of the former kernel's time, with them 0.2 to 0.6
+// of it), or where all rows run at once anyway.  Otherwise they cost up to 4 times the former kernel (2048 rows of
+// 10 genes, G(n, M) of 400000 nodes), the deletion bitmap alone 0.9.  Over 432 calls (G(n, M), BA, HK and R-MAT
+// graphs of 20000 to 700000 nodes, 256 to 2048 rows of 10 to 2000 genes, random and hub-heavy): 0.56 of the former
+// kernel's time on average, 1.03 at most; the better variant and thread count of each call give 0.55.
+// Threads: as many as let the rows that shared memory holds share an SM, more where rows are few; without the
+// bitmaps no more than there are genes (one warp takes 32).
+ResidShape resid_shape(const gapa_surrogate* s, int rows, int k) {
+    const gapa_ctx* c = s->ctx;
+    const size_t words = s->resid_smem / 4;
+    const size_t per_sm = std::max<size_t>(1, c->smem_per_sm / (3 * s->resid_smem + 14336));  // (12.4 KB static)
+    const size_t waves = ((size_t)rows + per_sm * c->num_sms - 1) / (per_sm * c->num_sms);
+    const bool tail = s->max_degree >= 128;
+    const double arcs = (double)k * s->mean_degree;
+    const bool dense = 2 * arcs >= (double)words;
+    ResidShape r;
+    r.once = s->resid_once &&
+             (waves == 1 || (dense && per_sm >= 2) || (tail && (per_sm >= 3 || waves <= 2)) ||
+              (tail && dense && (waves <= 4 || arcs >= (double)words)));
+    const size_t fit = r.once ? per_sm : std::max<size_t>(1, c->smem_per_sm / (s->resid_smem + 2048));
+    const size_t on_sm = ((size_t)rows + c->num_sms - 1) / c->num_sms;
+    size_t most = 1024;
+    if (!r.once) most = k <= 256 ? 256 : k <= 512 ? 512 : 1024;
+    size_t T = 256;
+    while (T < most && (2 * fit * T <= 2048 || on_sm * T < 2048)) T *= 2;
+    r.threads = (int)T;
+    return r;
+}
+
 // Features + forward; keeps the transposed copies for a training step.
 // Residual-degree counts of `rows` deletion sets into s->resid, standardised over those rows.
 int compute_resid(gapa_surrogate* s, const int32_t* pop, int rows, int k, cudaStream_t st) {
     if (rows <= 0) return GAPA_OK;
     ProfileScope prof(s->ctx, st, 2, 2);
-    // 256 threads per row where that fills the device's 2048 per SM, more where rows are few or their
-    // bitmaps keep CTAs off an SM (256 rows of 1500 genes, n = 30011: 102 us by the former per-arc kernel at 256 threads, 30 us at 1024)
-    const size_t smem = s->resid_once ? 3 * s->resid_smem : s->resid_smem;
-    const size_t per_sm = s->ctx->smem_per_sm / (smem + (s->resid_once ? 14336 : 10240));
-    int T = 256;
-    while (T < 1024 && (per_sm * T < 2048 || (long long)rows * T < 2048ll * s->ctx->num_sms)) T *= 2;
-    const auto kern = s->resid_once ? resid_kernel<true> : resid_kernel<false>;
-    kern<<<rows, T, smem, st>>>(pop, rows, k, s->n, s->low, s->nbr, s->row_ptr, s->col, s->resid, s->rsums, s->rstats);
+    const ResidShape shape = resid_shape(s, rows, k);
+    const auto kern = shape.once ? resid_kernel<true> : resid_kernel<false>;
+    kern<<<rows, shape.threads, (shape.once ? 3 : 1) * s->resid_smem, st>>>(pop, rows, k, s->n, s->low, s->nbr, s->row_ptr,
+                                                                            s->col, s->resid, s->rsums, s->rstats);
     resid_z_kernel<<<(rows + 127) / 128, 128, 0, st>>>(s->resid, rows, s->rstats);
     GAPA_CUDA(cudaGetLastError());
     return GAPA_OK;
@@ -1436,9 +1473,11 @@ int gapa_surrogate_create(gapa_surrogate** out, gapa_ctx* ctx, const gapa_surrog
         return bail(gapa_fail(GAPA_ERR_CUDA, "reading degrees"));
     std::vector<float> lg(s->n), dg(s->n);
     for (int v = 0; v < s->n; ++v) {
+        s->max_degree = std::max(s->max_degree, rp[v + 1] - rp[v]);
         dg[v] = (float)(rp[v + 1] - rp[v]);
         lg[v] = (float)std::log1p((double)dg[v]);
     }
+    s->mean_degree = (double)rp[s->n] / s->n;
     s->inv2E = ctx->g.num_edges > 0 ? (float)(1.0 / (2.0 * ctx->g.num_edges)) : 0.f;
     cudaMemcpy(s->logdeg, lg.data(), lg.size() * 4, cudaMemcpyHostToDevice);
     cudaMemcpy(s->deg, dg.data(), dg.size() * 4, cudaMemcpyHostToDevice);

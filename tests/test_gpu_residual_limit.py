@@ -1,4 +1,5 @@
-"""Residual counts of the largest graph whose deletion bitmap fits in shared memory."""
+"""Residual counts where the choice of kernel changes: the largest graph whose deletion bitmap fits in shared
+memory, and few or many genes and rows on graphs with long and with short adjacencies."""
 import numpy as np
 import pytest
 
@@ -33,3 +34,31 @@ def test_residual_counts_at_the_size_limit():
         ctx.graph_upload(big.row_ptr, big.col)
         with pytest.raises(GapaError):
             Surrogate(ctx, make_surrogate_config(batch=16, ring=16), seed=1)
+
+
+# with the once / twice bitmaps and without (few genes on graphs of short adjacencies, many rows), 256 to 1024
+# threads per row
+@pytest.mark.parametrize("n,rows,k", [(30000, 1300, 20), (30000, 1300, 700), (160000, 330, 40), (160000, 330, 1100),
+                                      (160000, 150, 40), (420000, 310, 600)])
+@pytest.mark.parametrize("shape", ["even", "hubs"])
+def test_residual_counts_by_either_kernel(n, rows, k, shape):
+    import torch
+
+    from paper_2412_20980_gb300 import Context, Surrogate, make_surrogate_config
+
+    rng = np.random.default_rng(n + k)
+    u, v = rng.integers(0, n, (2, int(1.6 * n)))
+    if shape == "hubs":
+        v[: n // 4] = rng.integers(0, 30, n // 4)
+    g = synth.csr_from_edges(n, u[u != v], v[u != v])
+    pop = np.stack([rng.permutation(n)[:k] for _ in range(8)]).astype(np.int32)
+    pop[::2, :8] = np.argsort(-np.diff(g.row_ptr), kind="stable")[:8]  # the longest adjacencies, some genes twice
+    pop[0, :2] = (-1, n)  # ignored
+    full = np.concatenate([pop] * (rows // 8 + 1))[:rows]
+    with Context(0) as ctx:
+        ctx.graph_upload(g.row_ptr, g.col)
+        sg = Surrogate(ctx, make_surrogate_config(batch=16, ring=16), seed=1)
+        got = sg.residual(torch.from_numpy(full).cuda()).cpu().numpy()
+        want = _counts(g, pop)
+        assert np.array_equal(got, np.concatenate([want] * (rows // 8 + 1))[:rows])
+        sg.close()
