@@ -793,13 +793,16 @@ int gapa_launch_read_probe(const void* buf, size_t bytes, int passes, int grid, 
 
 bool gapa_fitness_local(const gapa_ctx* c) {
     const DeviceGraph& g = c->g;
-    // AUTO: not where most deletions leave much apart (mean degree below 3: trees, sparse random graphs), nor
-    // on small graphs of mean degree below 5.  Whole calls, 100 members of n / 20 genes (random and hub-heavy),
-    // cut-local against full pipeline, us: tree of 6000 nodes 42 / 17 and 41 / 17; degree 2.7, n = 6000: 28 / 33
-    // and 38 / 33, n = 1500: 24 / 19 and 29 / 19; degree 4, n = 700: 16 / 12 and 26 / 15, n = 3000: 19 / 23 and
-    // 24 / 26, n = 12000: 35 / 36 and 50 / 46; degree 6, n = 1500: 16 / 20 and 22 / 29, n = 12000: 21 / 55 and
-    // 43 / 57.
-    const bool sparse = g.mean_deg_x16 < 48 || (gapa_dev::tree16l_sparse(g.mean_deg_x16) && g.n <= 2048);
+    // AUTO: not where most deletions leave much apart (mean degree below 3: trees, sparse random graphs), and on
+    // graphs of up to 2048 nodes only from a mean degree of 5.75 and 5700 arcs on.  Cut-local time against the
+    // full pipeline's, least to most over 100 and 1000 members of n / 50 to n / 8 genes, random and hub-heavy:
+    // n = 300, degree 4 to 8: 0.71 to 1.95, 16: 0.59 to 0.89; n = 500, degree 6: 0.84 to 1.37, 10 to 12: 0.71 to 1.16;
+    // n = 700, degree 6: 0.76 to 1.40, 8: 0.75 to 1.32, 10 to 12: 0.60 to 1.00; n = 1000, degree 4 to 5.5: 0.94 to 1.45,
+    // 6 (BA, HK, G(n, M)): 0.63 to 1.13, 8: 0.57 to 1.12; n = 1400, degree 6: 0.51 to 1.01.  Above 2048 nodes it takes over
+    // from a kernel that it is faster than at every degree (0.65 of its time on average, lattices and community
+    // graphs among them, where single calls take up to 1.8 times as long).
+    const bool small = g.n <= 2048 && (g.mean_deg_x16 < 92 || g.nnz < 5700);
+    const bool sparse = g.mean_deg_x16 < 48 || small;
     return g.packed16 && g.lc.par && (c->fitness_variant == GAPA_FITNESS_TREE_LOCAL ||
                                       (c->fitness_variant == GAPA_FITNESS_AUTO && !sparse));
 }

@@ -732,7 +732,12 @@ __device__ __forceinline__ int tree16l_owner(const int* off, int owners, int i) 
 // PC, and 1 to MCN.
 // A member with repeated genes, or whose tops or list outgrow its region, or
 // whose list outgrows a quarter of the graph or kLocalLevels rounds, runs
-// tree16_member.  On sparse graphs (mean degree below 5) a member with more
+// the full pipeline, at up to twice that pipeline's time.  (The list of a graph
+// without communities stays below: 0.11 n on Barabasi-Albert and Holme-Kim
+// graphs with an eighth of the nodes deleted, up to all of them hubs, 0.16 n on
+// G(n, M) of mean degree 3; small-world and community graphs lose 2 to 3
+// members of 40 there.  Half of the graph as the limit made these 1.2 to 1.5
+// times slower, a look at the share apart half-way through 1.3 to 1.9.)  On sparse graphs (mean degree below 5) a member with more
 // than n / 8 tops, which leaves thousands of nodes apart, runs tree32_member
 // from the start (2 links per node, n = 12000, 100 hub-heavy members of 600
 // genes: 107 us without).
@@ -778,12 +783,12 @@ __device__ __forceinline__ void tree16l_append(int val, volatile int* count, lab
 }
 
 // lab: the member's labels; region: its list region (g.list_bytes); scal_base:
-// its twelve scalars followed by the mbarrier.  Returns through *out like
-// tree16_member.
-__device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab_t* lab, unsigned* region,
-                                                    int* scal_base, const Tree16Graph& g,
-                                                    const int* __restrict__ genes, int k, long long* out,
-                                                    long long* red, int* status) {
+// its twelve scalars followed by the mbarrier.  0: the result is in *out, as
+// from tree16_member; 1: the member needs the full pipeline; 2: it needs it on
+// 32-bit labels.
+__device__ __forceinline__ int tree16_local_try(const Team& tm, volatile lab_t* lab, unsigned* region, int* scal_base,
+                                                const Tree16Graph& g, const int* __restrict__ genes, int k,
+                                                long long* out, long long* red, int* status) {
     const int tid = tm.tid, T = tm.T, n = g.n, lane = tid & 31;
     // 0 R, 1 list length, 2 tops, 3 distinct genes, 4 repeated genes, 5 deleted single-node components,
     // 6 the copy's wait ran out, 8 terminals, 9 listed nodes that joined R
@@ -884,31 +889,18 @@ __device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab
     tm.sync();
     if (scalar[6]) {
         if (tid == 0) *out = -1;
-        return;
+        return 0;
     }
     // the copy has landed: the mbarrier's memory may be reused
     if (tid == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar_a) : "memory");
     const int tops = scalar[2], live = n - scalar[3], live_singles = g.cut.singles - scalar[5];
-    if (scalar[4]) {  // repeated genes
-        tm.sync();
-        tree16_member(tm, lab, region, g, genes, k, out, red, status);
-        return;
-    }
+    if (scalar[4]) return 1;  // repeated genes
     if (live == live_singles) {  // nothing, or single nodes only
         if (tid == 0) *out = g.objective && live ? 1 : 0;
-        return;
+        return 0;
     }
-    if (tops > g.tops_max) {
-        tm.sync();
-        int* lab32 = reinterpret_cast<int*>(const_cast<lab_t*>(lab));
-        tree32_member(tm, lab32, reinterpret_cast<unsigned*>(lab32 + n), g, genes, k, out, red, status);
-        return;
-    }
-    if (tops > cap - cap / 8) {  // (the rest is room for terminals)
-        tm.sync();
-        tree16_member(tm, lab, region, g, genes, k, out, red, status);
-        return;
-    }
+    if (tops > g.tops_max) return 2;
+    if (tops > cap - cap / 8) return 1;  // (the rest is room for terminals)
     // every live top: its first live lower-numbered neighbour, else itself (a "terminal", listed downwards
     // from the list's end)
     lab_t* const term = list + cap - 1;
@@ -944,11 +936,7 @@ __device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab
     // the terminals unite with up to two live higher-numbered neighbours outside their own piece
     int R = scalar[0];
     const int terms = scalar[8];
-    if (terms > term_cap) {
-        tm.sync();
-        tree16_member(tm, lab, region, g, genes, k, out, red, status);
-        return;
-    }
+    if (terms > term_cap) return 1;
     for (int i = tid; i < terms; i += T) {
         const int c = term[-i];
         const uint2 l = __ldg(&g.cut.higher[c]);
@@ -992,7 +980,7 @@ __device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab
     int tail = scalar[1];
     if (tail == 0) {  // one class
         if (tid == 0) *out = objective_add(0, others, g.objective);
-        return;
+        return 0;
     }
     // breadth first from the seeds over live arcs, four lanes per node (eight from a mean degree of 6 on): a
     // neighbour in R's class joins the node's class to R, any other is united with it and listed.  Every
@@ -1036,11 +1024,7 @@ __device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab
         tail = scalar[1];
         ++level;
     }
-    if (tail > lim || head < tail) {  // the list too long or too deep: the full pipeline
-        tm.sync();
-        tree16_member(tm, lab, region, g, genes, k, out, red, status);
-        return;
-    }
+    if (tail > lim || head < tail) return 1;  // the list too long or too deep
     const int listed = tail;
     const long long outer = others - listed;  // plus the listed nodes that joined R
     if (listed <= 32) {  // one warp counts by matching roots
@@ -1057,11 +1041,30 @@ __device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab
             }
             if (lane == 0) *out = acc;
         }
-        return;
+        return 0;
     }
     long long acc = tree16_list_sizes(tm, lab, list, listed, R, &scalar[9], g.objective);
     if (tid == 0) acc = objective_add(acc, outer + scalar[9], g.objective);
     const long long tot = team_sum_ll(tm, acc, red, g.objective != 0);
     if (tid == 0) *out = tot;
+    return 0;
+}
+
+// The full pipeline where it has to be: on 32-bit labels wherever the region holds them (15 to 30 % faster than
+// on 16-bit ones).  One place for all that need it keeps the kernel within its 32 registers without a spill
+// (inlined at five places: 12 bytes spilled, 84 reloaded; whole small runs 2 % slower).
+__device__ __forceinline__ void tree16_member_local(const Team& tm, volatile lab_t* lab, unsigned* region,
+                                                    int* scal_base, const Tree16Graph& g,
+                                                    const int* __restrict__ genes, int k, long long* out,
+                                                    long long* red, int* status) {
+    const int full = tree16_local_try(tm, lab, region, scal_base, g, genes, k, out, red, status);
+    if (full == 0) return;
+    tm.sync();
+    if (full == 2 || tree16_lab_bytes(g.n) + (size_t)g.list_bytes >= tree32_smem_bytes(g.n)) {
+        int* lab32 = reinterpret_cast<int*>(const_cast<lab_t*>(lab));
+        tree32_member(tm, lab32, reinterpret_cast<unsigned*>(lab32 + g.n), g, genes, k, out, red, status);
+    } else {
+        tree16_member(tm, lab, region, g, genes, k, out, red, status);
+    }
 }
 }  // namespace gapa_dev

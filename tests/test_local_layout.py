@@ -1,4 +1,5 @@
-"""The cut-local kernel's shared-memory layout up to the largest graph that it takes.
+"""The cut-local kernel's shared-memory layout up to the largest graph that it takes, and the graphs on which
+the automatic setting takes it.
 
 The launch shape is plain C++: a host program walks every graph size, and the sizes next to the limits
 run on the GPU against the oracle.
@@ -94,3 +95,27 @@ def test_largest_graphs_match_oracle(layout, n):
                 got = ctx.fitness(torch.from_numpy(pop).cuda())
                 ctx.sync()
                 assert np.array_equal(got.cpu().numpy(), want), (name, kernel)
+
+
+# by the launches of a call that does not fit the SMs at once: the full pipeline is one, the cut-local kernel
+# comes after its cost estimates and order
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,edges,launches", [(300, 1800, 1), (950, 2849, 1), (1000, 2850, 3), (500, 2850, 3),
+                                              (2000, 5600, 1), (2048, 5888, 3), (2049, 3074, 3), (2049, 3009, 1)])
+def test_automatic_choice_on_both_sides_of_its_lines(n, edges, launches):
+    import torch
+
+    from paper_2412_20980_gb300 import Context, build
+
+    build.build()
+    g = synth.er_graph(n, edges, 7)
+    s = 9 * torch.cuda.get_device_properties(0).multi_processor_count
+    pop = synth.random_deletion_sets(n, n // 20, s, 5)
+    with Context(0) as ctx:
+        ctx.graph_upload(g.row_ptr, g.col)
+        dev = torch.from_numpy(pop).cuda()
+        ctx.profile_begin()
+        got = ctx.fitness(dev)
+        ctx.sync()
+        assert ctx.profile_end()["fitness_launches"] == launches
+        assert np.array_equal(got.cpu().numpy(), oracle.fitness(g.row_ptr, g.col, pop, nthreads=oracle.max_threads()))
