@@ -29,6 +29,15 @@ struct DeviceGuard {
     }
 };
 
+void free_piece(PieceTables& t) {
+    DeviceForest& a = t.alt;
+    void* ptrs[] = {t.kids, t.roots, t.cut, t.sz, t.pre, t.at, t.crep, t.nroot, t.csize,
+                    a.perm, a.tparent, a.palt, a.lo_ptr, a.lo_col, a.kids, a.roots, a.cut, a.fptr, a.fcol16,
+                    a.nontree, a.sz, a.pre, a.at, a.crep, a.nroot, a.csize};
+    for (void* q : ptrs) cudaFree(q);
+    t = PieceTables();
+}
+
 void free_graph(DeviceGraph& g) {
     cudaFree(g.row_ptr);
     cudaFree(g.col);
@@ -36,22 +45,10 @@ void free_graph(DeviceGraph& g) {
     cudaFree(g.probe);
     cudaFree(g.perm);
     cudaFree(g.tparent);
-    cudaFree(g.kids);
-    cudaFree(g.roots);
-    cudaFree(g.cut);
     cudaFree(g.order);
-    cudaFree(g.sz);
-    cudaFree(g.pre);
-    cudaFree(g.at);
-    cudaFree(g.crep);
-    cudaFree(g.nroot);
-    cudaFree(g.csize);
+    free_piece(g.piece);
     void* cut_ptrs[] = {g.lc.par, g.lc.gene, g.lc.lower, g.lc.higher, g.lc.near, g.lc.roots, g.lc.cost};
     for (void* q : cut_ptrs) cudaFree(q);
-    DeviceForest& a = g.alt;
-    void* alt_ptrs[] = {a.perm, a.tparent, a.palt, a.lo_ptr, a.lo_col, a.kids, a.roots, a.cut, a.fptr, a.fcol16,
-                        a.nontree, a.sz, a.pre, a.at, a.crep, a.nroot, a.csize};
-    for (void* q : alt_ptrs) cudaFree(q);
     cudaFree(g.nontree);
     cudaFree(g.fptr);
     cudaFree(g.fcol16);
@@ -379,6 +376,63 @@ int upload_forest(const ForestHost& f, int32_t n, DeviceForest& d) {
     return GAPA_OK;
 }
 
+// Children of every node as (first, count, 0, 0), which BFS numbers consecutively; false if some are not.
+bool children_ranges(const std::vector<int32_t>& tparent, std::vector<int4>& kids) {
+    const int32_t n = (int32_t)tparent.size();
+    kids.resize((size_t)n);
+    for (int32_t b = 0; b < n; ++b) kids[b] = make_int4(b, 0, 0, 0);
+    for (int32_t x = 0; x < n; ++x) {
+        const int32_t p = tparent[x];
+        if (p == x) continue;
+        if (kids[p].y == 0) kids[p].x = x;
+        else if (kids[p].x + kids[p].y != x) return false;
+        kids[p].y += 1;
+    }
+    return true;
+}
+
+// Tables of the forest-piece kernel (see PieceTables) from the BFS forest and the graph (rows by original id).
+int upload_piece_tables(const BfsForest& bf, const std::vector<int32_t>& rp, const std::vector<int32_t>& col, int32_t n,
+                        PieceTables& t) {
+    std::vector<int4> kids;
+    if (!children_ranges(bf.tparent, kids)) return GAPA_OK;
+    // cost estimate of deleting node b: the nodes below those children of b whose only lower
+    // neighbour is b (they become roots of pieces to be listed)
+    std::vector<int32_t> below((size_t)n, 1), cut((size_t)n, 0), cut_by_id((size_t)n);
+    for (int32_t v = n - 1; v >= 0; --v)
+        if (bf.tparent[v] != v) below[bf.tparent[v]] += below[v];
+    for (int32_t v = 0; v < n; ++v)
+        if (bf.tparent[v] != v && bf.lo_ptr[v + 1] - bf.lo_ptr[v] == 1) cut[bf.tparent[v]] += below[v];
+    for (int32_t v = 0; v < n; ++v) cut_by_id[v] = cut[bf.perm[v]];  // indexed by original node id
+    const ForestIntervals fi = forest_intervals(bf.tparent, bf.lo_ptr, bf.lo_col);
+    auto up = [](void** dst, const void* src, size_t bytes) {
+        return cudaMalloc(dst, std::max<size_t>(bytes, 16)) == cudaSuccess &&
+               (bytes == 0 || cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess);
+    };
+    if (!(up((void**)&t.kids, kids.data(), sizeof(int4) * (size_t)n) && up((void**)&t.cut, cut_by_id.data(), 4 * (size_t)n) &&
+          up((void**)&t.roots, bf.roots.data(), 4 * bf.roots.size()) && up((void**)&t.sz, fi.sz.data(), 4 * (size_t)n) &&
+          up((void**)&t.pre, fi.pre.data(), 4 * (size_t)n) && up((void**)&t.at, fi.at.data(), 2 * (size_t)n) &&
+          up((void**)&t.crep, fi.crep.data(), 4 * (size_t)n) && up((void**)&t.nroot, fi.nroot.data(), 4 * (size_t)n) &&
+          up((void**)&t.csize, fi.csize.data(), 4 * (size_t)n))) {
+        cudaGetLastError();
+        return gapa_fail(GAPA_ERR_OOM, "forest-piece tables of %d nodes", n);
+    }
+    t.num_roots = (int)bf.roots.size();
+    t.tree_pc = fi.tree_pc;
+    // the second forest, numbered with the top hubs last (about 0.5 % of the nodes, 8 to 256)
+    const int hubs = std::max(8, std::min(256, n / 200));
+    if (n > 4 * hubs) {
+        const ForestHost fb = forest_host(n, rp, col, hub_last_perm(n, rp, col, hubs));
+        if (fb.ok) {
+            const int rc = upload_forest(fb, n, t.alt);
+            if (rc != GAPA_OK) return rc;
+            t.has_alt = true;
+        }
+    }
+    t.ready = true;
+    return GAPA_OK;
+}
+
 // Tables of the cut-local kernel (see CutTables) from the BFS forest, the graph (rows by original id)
 // and the children ranges by number.
 int upload_cut_tables(const BfsForest& bf, const std::vector<int32_t>& rp, const std::vector<int32_t>& col, int32_t n,
@@ -607,6 +661,23 @@ int ensure_stage(gapa_ctx* c, size_t pop_elems, size_t fit_elems) {
 
 GaParams gapa_make_params(gapa_ctx* c, const gapa_config* cfg, int g, const int* g_ptr) {
     return make_params(c, cfg, g, g_ptr);
+}
+
+int gapa_piece_prepare(gapa_ctx* c) {
+    DeviceGraph& g = c->g;
+    if (g.n <= 0 || !g.lc.par || g.piece.ready) return GAPA_OK;
+    // not inside a capture: the full pipeline takes the calls then, with the same results
+    cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &state) != cudaSuccess || state != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return GAPA_OK;
+    }
+    std::vector<int32_t> rp((size_t)g.n + 1), col((size_t)g.nnz);
+    GAPA_CUDA(cudaMemcpy(rp.data(), g.row_ptr, 4 * rp.size(), cudaMemcpyDeviceToHost));
+    if (g.nnz) GAPA_CUDA(cudaMemcpy(col.data(), g.col, 4 * col.size(), cudaMemcpyDeviceToHost));
+    const int rc = upload_piece_tables(bfs_forest(g.n, rp, col), rp, col, g.n, g.piece);
+    if (rc != GAPA_OK) free_piece(g.piece);
+    return rc;
 }
 
 // Validation and buffers of a whole run (outside any capture).
@@ -984,77 +1055,17 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     GAPA_CUDA(cudaMemcpy(g.perm, bf.perm.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
     GAPA_CUDA(cudaMemcpy(g.tparent, bf.tparent.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
     if (g.packed16) {
-        // cut-local TREE kernel and forest-piece kernel: children ranges (consecutive in BFS order) and
-        // component roots
-        std::vector<int4> kids((size_t)n);
-        bool contiguous = true;
-        for (int32_t b = 0; b < n; ++b) kids[b] = make_int4(b, 0, 0, 0);
-        for (int32_t x = 0; x < n && contiguous; ++x) {
-            const int32_t p = bf.tparent[x];
-            if (p == x) continue;
-            if (kids[p].y == 0) kids[p].x = x;
-            else if (kids[p].x + kids[p].y != x) contiguous = false;
-            kids[p].y += 1;
-        }
-        if (contiguous && gapa_dev::local_admits(n, g.mean_deg_x16, c->fit_smem_max)) {
+        std::vector<int4> kids;
+        if (children_ranges(bf.tparent, kids) && gapa_dev::local_admits(n, g.mean_deg_x16, c->fit_smem_max)) {
             const int lrc = upload_cut_tables(bf, rp, sorted, n, kids, g.lc);
             if (lrc != GAPA_OK) {
                 free_graph(g);
                 return lrc;
             }
-            // cost estimate of deleting node b: the nodes below those children of b whose only lower
-            // neighbour is b (they become roots of pieces to be listed)
-            std::vector<int32_t> below((size_t)n, 1), cut((size_t)n, 0);
-            for (int32_t v = n - 1; v >= 0; --v)
-                if (bf.tparent[v] != v) below[bf.tparent[v]] += below[v];
-            for (int32_t v = 0; v < n; ++v)
-                if (bf.tparent[v] != v && bf.lo_ptr[v + 1] - bf.lo_ptr[v] == 1) cut[bf.tparent[v]] += below[v];
-            if (cudaMalloc(&g.kids, sizeof(int4) * std::max<size_t>((size_t)n, 1)) != cudaSuccess ||
-                cudaMalloc(&g.cut, sizeof(int32_t) * std::max<size_t>((size_t)n, 1)) != cudaSuccess ||
-                cudaMalloc(&g.order, sizeof(int32_t) * (5 * (size_t)kOrderCap + 16)) != cudaSuccess ||
-                cudaMalloc(&g.roots, sizeof(int32_t) * std::max<size_t>(bf.roots.size(), 1)) != cudaSuccess) {
+            if (cudaMalloc(&g.order, sizeof(int32_t) * (5 * (size_t)kOrderCap + 16)) != cudaSuccess) {
                 free_graph(g);
                 cudaGetLastError();
-                return gapa_fail(GAPA_ERR_OOM, "children ranges of %d nodes", n);
-            }
-            GAPA_CUDA(cudaMemcpy(g.kids, kids.data(), sizeof(int4) * (size_t)n, cudaMemcpyHostToDevice));
-            std::vector<int32_t> cut_by_id((size_t)n);  // indexed by original node id
-            for (int32_t v = 0; v < n; ++v) cut_by_id[v] = cut[bf.perm[v]];
-            GAPA_CUDA(cudaMemcpy(g.cut, cut_by_id.data(), sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice));
-            if (!bf.roots.empty())
-                GAPA_CUDA(cudaMemcpy(g.roots, bf.roots.data(), sizeof(int32_t) * bf.roots.size(),
-                                     cudaMemcpyHostToDevice));
-            g.num_roots = (int)bf.roots.size();
-            {
-                // subtree intervals of the forest-piece kernel
-                const ForestIntervals fi = forest_intervals(bf.tparent, bf.lo_ptr, bf.lo_col);
-                auto up = [](void** dst, const void* src, size_t bytes) {
-                    return cudaMalloc(dst, std::max<size_t>(bytes, 16)) == cudaSuccess &&
-                           cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
-                };
-                if (!(up((void**)&g.sz, fi.sz.data(), 4 * (size_t)n) && up((void**)&g.pre, fi.pre.data(), 4 * (size_t)n) &&
-                      up((void**)&g.at, fi.at.data(), 2 * (size_t)n) &&
-                      up((void**)&g.crep, fi.crep.data(), 4 * (size_t)n) &&
-                      up((void**)&g.nroot, fi.nroot.data(), 4 * (size_t)n) &&
-                      up((void**)&g.csize, fi.csize.data(), 4 * (size_t)n))) {
-                    free_graph(g);
-                    cudaGetLastError();
-                    return gapa_fail(GAPA_ERR_OOM, "subtree intervals of %d nodes", n);
-                }
-                g.tree_pc = fi.tree_pc;
-            }
-            // the second forest, numbered with the top hubs last (about 0.5 % of the nodes, 8 to 256)
-            const int hubs = std::max(8, std::min(256, n / 200));
-            if (n > 4 * hubs) {
-                const ForestHost fb = forest_host(n, rp, sorted, hub_last_perm(n, rp, sorted, hubs));
-                if (fb.ok) {
-                    int frc = upload_forest(fb, n, g.alt);
-                    if (frc != GAPA_OK) {
-                        free_graph(g);
-                        return frc;
-                    }
-                    g.has_alt = true;
-                }
+                return gapa_fail(GAPA_ERR_OOM, "member order of the cut-local kernel");
             }
         }
     }
@@ -1131,7 +1142,10 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     }
     c->g = g;
     c->sp_refused = gapa_dev::kSpShapes;  // room may have come back
-    return GAPA_OK;
+    if (c->fitness_variant != GAPA_FITNESS_PIECE) return GAPA_OK;
+    const int prc = gapa_piece_prepare(c);
+    if (prc != GAPA_OK) free_graph(c->g);
+    return prc;
 }
 
 int gapa_pop_init(gapa_ctx* c, const gapa_config* cfg, int32_t* pop_dev) {
@@ -1318,6 +1332,11 @@ int gapa_set_fitness_kernel(gapa_ctx* c, int variant) {
     if (!c) return gapa_fail(GAPA_ERR_INVALID_ARG, "ctx is NULL");
     if (variant < GAPA_FITNESS_AUTO || variant > GAPA_FITNESS_SPARSE)
         return gapa_fail(GAPA_ERR_INVALID_ARG, "unknown fitness kernel %d", variant);
+    if (variant == GAPA_FITNESS_PIECE) {
+        DeviceGuard guard(c->device);
+        const int rc = gapa_piece_prepare(c);
+        if (rc != GAPA_OK) return rc;
+    }
     c->fitness_variant = variant;
     return GAPA_OK;
 }

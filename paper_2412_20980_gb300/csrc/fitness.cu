@@ -650,7 +650,7 @@ gapa_dev::PieceGraph piece_graph(const gapa_ctx* c, bool second) {
     const DeviceGraph& g = c->g;
     gapa_dev::PieceGraph p{};
     p.n = g.n;
-    p.tree_pc = g.tree_pc;
+    p.tree_pc = g.piece.tree_pc;
     p.objective = c->objective;
     if (!second) {
         p.perm = g.perm;
@@ -660,17 +660,17 @@ gapa_dev::PieceGraph piece_graph(const gapa_ctx* c, bool second) {
         p.lo_col = g.lo_col;
         p.fptr = g.fptr;
         p.fcol = g.fcol16;
-        p.kids = g.kids;
-        p.sz = g.sz;
-        p.pre = g.pre;
-        p.at = g.at;
-        p.crep = g.crep;
-        p.nroot = g.nroot;
-        p.csize = g.csize;
-        p.roots = g.roots;
-        p.num_roots = g.num_roots;
+        p.kids = g.piece.kids;
+        p.sz = g.piece.sz;
+        p.pre = g.piece.pre;
+        p.at = g.piece.at;
+        p.crep = g.piece.crep;
+        p.nroot = g.piece.nroot;
+        p.csize = g.piece.csize;
+        p.roots = g.piece.roots;
+        p.num_roots = g.piece.num_roots;
     } else {
-        const DeviceForest& a = g.alt;
+        const DeviceForest& a = g.piece.alt;
         p.perm = a.perm;
         p.tparent = a.tparent;
         p.palt = a.palt;
@@ -710,14 +710,14 @@ int launch_piece(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, in
     int* defer = c->g.order + 4 * kOrderCap;
     int* ctl = defer + kOrderCap;
     if (!est_in) {
-        local_cost_kernel<<<s, 128, 0, st>>>(pop, k, n, c->g.cut, c->g.has_alt ? c->g.alt.cut : nullptr, e1, e2);
+        local_cost_kernel<<<s, 128, 0, st>>>(pop, k, n, c->g.piece.cut, c->g.piece.has_alt ? c->g.piece.alt.cut : nullptr, e1, e2);
         if (kernels) *kernels += 1;
     }
     const unsigned* a = est_in ? est_in : e1;
     piece_order_kernel<<<1, 1024, 0, st>>>(a, a + kOrderCap, s, c->g.order, est_min, ctl);
     PieceArgs pa;
     pa.g1 = piece_graph(c, false);
-    pa.g2 = c->g.has_alt ? piece_graph(c, true) : pa.g1;
+    pa.g2 = c->g.piece.has_alt ? piece_graph(c, true) : pa.g1;
     pa.L = L;
     const int grid = std::max(2, std::min(c->num_sms, (s + kPieceTeams - 1) / kPieceTeams));
     const size_t bytes = parents + (size_t)kPieceTeams * L.bytes;
@@ -810,7 +810,7 @@ static bool local_selected(const gapa_ctx* c) { return gapa_fitness_local(c); }
 
 // The forest-piece kernel: by request only (it needs the cut-local kernel's forests and cost tables).
 static bool piece_selected(const gapa_ctx* c) {
-    return c->g.packed16 && c->g.lc.par && c->g.sz && c->fitness_variant == GAPA_FITNESS_PIECE;
+    return c->g.packed16 && c->g.lc.par && c->g.piece.ready && c->fitness_variant == GAPA_FITNESS_PIECE;
 }
 
 bool gapa_fitness_uses_estimates(const gapa_ctx* c, int s) {
@@ -821,8 +821,8 @@ bool gapa_fitness_uses_estimates(const gapa_ctx* c, int s) {
 
 void gapa_estimate_tables(const gapa_ctx* c, const int** first, const int** second) {
     const bool piece = piece_selected(c);
-    *first = piece ? c->g.cut : c->g.lc.cost;
-    *second = piece && c->g.has_alt ? c->g.alt.cut : nullptr;
+    *first = piece ? c->g.piece.cut : c->g.lc.cost;
+    *second = piece && c->g.piece.has_alt ? c->g.piece.alt.cut : nullptr;
 }
 
 unsigned* gapa_estimate_buffer(gapa_ctx* c) { return reinterpret_cast<unsigned*>(c->g.order + kOrderCap); }

@@ -95,7 +95,7 @@ __device__ __forceinline__ int uniform_below(uint32_t x, int n) { return (int)__
 // neighbour when that one is lower), for the forest-piece kernel.
 struct DeviceForest {
     int* perm = nullptr;             // [n] original id -> number
-    int* tparent = nullptr;          // [n rounded up to 4]
+    int* tparent = nullptr;          // [n]
     int2* palt = nullptr;            // [n] (parent, second lower-numbered neighbour or -1)
     int* lo_ptr = nullptr;           // [n+1] lower-numbered neighbours (CSR, ascending)
     int* lo_col = nullptr;
@@ -159,6 +159,31 @@ struct CutTables {
     int* cost = nullptr;            // by original id: children + 1 (the member cost estimate sums it)
 };
 
+// Tables of the forest-piece kernel beside the BFS forest, made when that kernel is chosen.
+struct PieceTables {
+    bool ready = false;
+    int4* kids = nullptr;       // [n] children: x .. x+y-1, then z+y .. z+y+w-1 (a second run; w = 0 here,
+                                //     where children have consecutive numbers)
+    int* roots = nullptr;       // [num_roots] BFS number of every component's root
+    int num_roots = 0;
+    int* cut = nullptr;         // [n] per original node id: nodes below those of its tree children that
+                                //     have no other lower neighbour (deleting it alone cuts them off)
+    // per forest: the subtree size of every node, its position in a preorder walk (children in
+    // ascending order, roots in ascending order; a subtree is the interval [pre, pre + sz)), the
+    // node at each preorder position, the smallest root of every node's component (its
+    // representative), the next root of the same component (-1: none) and the component's size (at
+    // the representative)
+    int* sz = nullptr;
+    int* pre = nullptr;
+    unsigned short* at = nullptr;
+    int* crep = nullptr;
+    int* nroot = nullptr;
+    int* csize = nullptr;
+    long long tree_pc = 0;      // sum over the components of G of C(size, 2)
+    DeviceForest alt;           // the forest numbered with the top hubs last
+    bool has_alt = false;
+};
+
 struct DeviceGraph {
     int n = 0;
     long long nnz = 0;        // arcs = 2E
@@ -172,31 +197,12 @@ struct DeviceGraph {
     // order from the highest-degree node of each component, so every tree
     // parent has a smaller number than its child.
     int* perm = nullptr;        // [n] original id -> BFS number
-    int* tparent = nullptr;     // [n rounded up to 4] BFS number -> BFS number of its tree parent (roots: itself)
-    int4* kids = nullptr;       // [n] children: x .. x+y-1, then z+y .. z+y+w-1 (a second run; w = 0 here,
-                                //     where children have consecutive numbers)
-    int* roots = nullptr;       // [num_roots] BFS number of every component's root
-    int num_roots = 0;
+    int* tparent = nullptr;     // BFS number -> BFS number of its tree parent (roots: itself)
     CutTables lc;               // cut-local TREE kernel (lc.par null: not on this graph)
-    int* cut = nullptr;         // [n] per original node id: nodes below those of its tree children that
-                                //     have no other lower neighbour (deleting it alone cuts them off)
-    int* order = nullptr;       // [5 * kOrderCap + 16] the members, costliest first (bit 30: use `alt`), then
-                                //     their cost estimates under this forest, under `alt`, and the lower,
+    int* order = nullptr;       // [5 * kOrderCap + 16] the members, costliest first (bit 30: use `piece.alt`), then
+                                //     their cost estimates under this forest, under the other, and the lower,
                                 //     then the members deferred by the forest-piece kernel and their count
-    DeviceForest alt;           // the forest numbered with the top hubs last (forest-piece kernel only)
-    // forest-piece kernel, per forest: the subtree size of every node, its position in a preorder
-    // walk (children in ascending order, roots in ascending order; a subtree is the interval
-    // [pre, pre + sz)), the node at each preorder position, the smallest root of every node's
-    // component (its representative), the next root of the same component (-1: none) and the
-    // component's size (at the representative)
-    int* sz = nullptr;
-    int* pre = nullptr;
-    unsigned short* at = nullptr;
-    int* crep = nullptr;
-    int* nroot = nullptr;
-    int* csize = nullptr;
-    long long tree_pc = 0;      // sum over the components of G of C(size, 2)
-    bool has_alt = false;
+    PieceTables piece;          // forest-piece kernel (once that kernel is chosen)
     int* lo_ptr = nullptr;      // [n+1] CSR of lower-numbered neighbours (BFS numbers, ascending;
     int* lo_col = nullptr;      //        the first one is the tree parent)
     int2* palt = nullptr;       // [n] (tree parent, second lower-numbered neighbour or -1)
@@ -375,6 +381,8 @@ struct BatchPacket {
     int b, i0, cnt, teams;
 };
 
+// The forest-piece kernel's tables for the uploaded graph (nothing on graphs that kernel does not take).
+int gapa_piece_prepare(gapa_ctx* c);
 int gapa_launch_fitness(gapa_ctx* c, const int32_t* pop, int s, int k, int64_t* fit, cudaStream_t st,
                         const unsigned* est = nullptr);
 // True when gapa_launch_fitness runs the cut-local TREE kernel on this context (which then uses
