@@ -126,6 +126,7 @@ def graphs(workload: str):
 # R-MAT scale of the large workload (20; smaller only for profiling captures, --rmat-scale):
 # 16 edges per node, k = 10000 scaled with the node count
 RMAT_SCALE = [20]
+SIXDST_HOPS = 6
 
 
 def large_k() -> int:
@@ -183,10 +184,11 @@ def measured_peaks():
 # (fitness.cu and its headers) and, for graphs whose labels exceed shared memory, the sparse
 # kernel (fitness_sparse.cu, dispatched from fitness.cu)
 TRAFFIC_SOURCES = {
-    "large": ("fitness.cu", "fitness_sparse.cu", "tree16.cuh", "gapa_internal.cuh"),
-    "surrogate": ("fitness.cu", "fitness_sparse.cu", "tree16.cuh", "gapa_internal.cuh"),
+    "large": ("fitness.cu", "fitness_sparse.cu", "tree16.cuh", "local_layout.cuh", "sparse_layout.cuh", "gapa_internal.cuh"),
+    "surrogate": ("fitness.cu", "fitness_sparse.cu", "tree16.cuh", "local_layout.cuh", "sparse_layout.cuh",
+                  "gapa_internal.cuh"),
 }
-DEFAULT_TRAFFIC_SOURCES = ("fitness.cu", "tree16.cuh", "gapa_internal.cuh")
+DEFAULT_TRAFFIC_SOURCES = ("fitness.cu", "tree16.cuh", "local_layout.cuh", "gapa_internal.cuh")
 
 
 KERNEL_TEXT = {
@@ -473,6 +475,7 @@ def run_gapa(args, env: Env, gs):
             from paper_2412_20980_gb300.gapa import OBJECTIVE_SIXDST_PC
 
             c.set_objective(OBJECTIVE_SIXDST_PC)
+            c.set_sixdst_hops(SIXDST_HOPS)
         pa = c.pop_init(cfg)
         fa = c.fitness(pa)
         state.append([pa, fa, torch.empty_like(pa), torch.empty_like(fa)])
@@ -542,16 +545,18 @@ def run_gapa(args, env: Env, gs):
         # 1000-node graph is launch- and latency-bound, graded by generations per second
         fit_launches = 0
     if fit_launches and wl == "sixdst":
-        # bound by shared-memory gathers: 16 bytes per arc and node, 128-column strip and hop after the first
-        n_, hops = int(gs[0].n), 6
-        gather = (2 * int(gs[0].num_edges) + n_) * ((n_ + 127) // 128) * 16 * (hops - 1)
+        # bound by shared-memory gathers: one per arc and node, strip of columns and hop after the first.  The
+        # bytes are an upper bound: a strip stops at the first hop that changes nothing.
+        n_ = int(gs[0].n)
+        width = 128 if 32 * (n_ + 1) + 4 * ((n_ + 31) // 32) <= 230000 else 64  # columns of a strip
+        gather = (2 * int(gs[0].num_edges) + n_) * ((n_ + width - 1) // width) * width // 8 * (SIXDST_HOPS - 1)
         props = torch.cuda.get_device_properties(dev)
         peak = props.multi_processor_count * 128 * 2.07  # GB/s
         achieved = gather * fit_evals / (fit_ms / 1000.0) / 1e9
         roofline = {"bound": "shared memory", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": None,
-                    "kernel": "sdst_bits_kernel (bit rows of 128 columns in shared memory, one gather per arc and hop)",
-                    "bytes_per_eval": gather, "evals": fit_evals, "fitness_ms": fit_ms,
+                    "kernel": f"sdst_bits_kernel (bit rows of {width} columns in shared memory, one gather per arc and hop)",
+                    "bytes_per_eval": gather, "bytes_are": "an upper bound: every strip counted with all hops", "evals": fit_evals, "fitness_ms": fit_ms,
                     "peak_source": "nominal: 128 bytes per SM and clock at 2070 MHz",
                     "fitness_share_of_step": fit_ms / max(1e-9, total_ms)}
     elif fit_launches:
