@@ -175,7 +175,7 @@ int gapa_run(gapa_ctx* ctx, const gapa_config* cfg, int32_t* best_set_host, int6
  * graph and replayed.  Every instance's trajectory, final population and best
  * set equal those of gapa_run() on its own context and configuration.
  * Limits: every graph must fit the shared-memory fitness path (at most
- * ~57,000 nodes; GAPA_ERR_INVALID_ARG otherwise); all contexts on one device;
+ * ~55,800 nodes; GAPA_ERR_INVALID_ARG otherwise); all contexts on one device;
  * the batch borrows the contexts (they must outlive it) and runs on the first
  * context's stream. */
 typedef struct gapa_batch gapa_batch;
@@ -296,14 +296,14 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * ones), and only the classes left apart from the first live node's are listed
  * and searched; a member with repeated genes, or whose lists outgrow the
  * kernel's shared memory, takes the TREE path.  It needs a graph whose 16-bit
- * ids and labels fit in shared memory (n up to about 56,000 on GB300).
+ * ids and labels fit in shared memory (n up to 56,281 on GB300).
  * SAMPLED joins every live node to its first two live neighbours, takes the
  * tree of the highest-degree live node as the giant tree and lets only nodes
  * outside it scan their whole adjacency; EDGES runs union-find over every
  * undirected edge.  AUTO (the default) is TREE_LOCAL where it applies and the
  * mean degree is at least 3 (up to 2048 nodes: 5.75, with 5700 arcs or more),
  * else TREE.  Where the labels
- * do not fit in shared memory (n above about 56,000 on GB300), AUTO runs SPARSE
+ * do not fit in shared memory (n above 56,281 on GB300), AUTO runs SPARSE
  * (below), the TREE settings run the same phases on labels in global memory,
  * eight members interleaved per 32-byte sector, and EDGES and SAMPLED run one
  * CTA per member over a global label array. */

@@ -220,7 +220,7 @@ ForestIntervals forest_intervals(const std::vector<int32_t>& tparent, const std:
     return fi;
 }
 
-// The forest of a numbering `perm` (host side, n <= 65536): every node's
+// The forest of a numbering `perm` (host side, 16-bit ids): every node's
 // parent is its lowest-numbered neighbour when that one is lower (a root
 // otherwise), so parents precede children.  `ok` is false when some node's
 // children do not fall into at most two runs of consecutive numbers.
@@ -1040,7 +1040,7 @@ int gapa_graph_upload(gapa_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     g.num_nontree = (int)bf.nontree.size();
     g.mean_deg_x16 = n > 0 ? (int)((16 * nnz + n - 1) / n) : 0;
     // 16-bit ids only on the shared-memory path (labels + deleted-node bitmap)
-    // (the limit: 4 bytes per node, a bitmap and four scalars within a block's shared memory, n <= about 56,280)
+    // (the limit: 4 bytes per node, a bitmap and four scalars within a block's shared memory, n <= 56,281)
     g.packed16 = n < gapa_dev::kDead16 && gapa_dev::tree32_smem_bytes(n) <= c->fit_smem_max;
     const size_t nt_bytes = (g.packed16 ? 4 : 8) * std::max<size_t>(bf.nontree.size(), 4);
     if (cudaMalloc(&g.perm, sizeof(int32_t) * (size_t)n) != cudaSuccess ||

@@ -90,7 +90,7 @@ __device__ __forceinline__ int uniform_below(uint32_t x, int n) { return (int)__
 // ---------------------------------------------------------------------------
 // Context
 // ---------------------------------------------------------------------------
-// A second spanning forest of a graph with n <= 65536, in its own numbering
+// A second spanning forest of a graph with 16-bit ids, in its own numbering
 // (parents precede children; a node's parent is its lowest-numbered
 // neighbour when that one is lower), for the forest-piece kernel.
 struct DeviceForest {
@@ -212,7 +212,7 @@ struct DeviceGraph {
     unsigned short* fcol16 = nullptr;   // [2E]
     int* fcol32 = nullptr;              // [2E] the same with 32-bit ids (graphs that are not packed16)
     int mean_deg_x16 = 0;               // 16 * 2E / n, rounded up
-    bool packed16 = false;      // n <= 65536
+    bool packed16 = false;      // 16-bit ids: tree32_smem_bytes(n) within one block (n <= 56,281 on GB300)
     int bfs_depth = 0;          // largest BFS level
     // sparse fitness kernel (any n; sp_nforests = 0 when a BFS forest's children are not consecutive):
     // forest 0 on G itself (borrowing the arrays above), and forests of G with every edge of the top

@@ -1,9 +1,10 @@
-// Shared-memory TREE fitness pipelines for graphs of at most 65535 nodes with
-// 16-bit labels, written for a "team": a group of warps of one CTA that
-// evaluates one population member with its own slice of shared memory and its
-// own named barrier.  A whole CTA is one team (barrier 0); the batched
-// persistent kernel splits a CTA into 2, 4 or 8 teams so that small graphs run
-// several members per CTA.
+// Shared-memory TREE fitness pipelines with 16-bit ids (graphs of up to 56,281
+// nodes: the 32-bit labels and bitmap of the full pipeline within one block),
+// written for a "team": a group of warps of one CTA that evaluates one
+// population member with its own slice of shared memory and its own named
+// barrier.  A whole CTA is one team (barrier 0); the batched persistent kernel
+// splits a CTA into 2, 4 or 8 teams so that small graphs run several members
+// per CTA.
 //
 // Fitness (Section III-C, Eq. 13; PC(G) of Table "Whole"): pairwise
 // connectivity of G with the member's genes deleted.  Nodes are in BFS
