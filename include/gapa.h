@@ -301,8 +301,8 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * tree of the highest-degree live node as the giant tree and lets only nodes
  * outside it scan their whole adjacency; EDGES runs union-find over every
  * undirected edge.  AUTO (the default) is TREE_LOCAL where it applies and the
- * mean degree is at least 3 (up to 2048 nodes: 5.75, with 5700 arcs or more),
- * else TREE.  Where the labels
+ * mean degree is at least 3 (up to 2048 nodes: 5.75, with 5700 arcs, or 650
+ * nodes and a degree of eight times the mean), else TREE.  Where the labels
  * do not fit in shared memory (n above 56,281 on GB300), AUTO runs SPARSE
  * (below), the TREE settings run the same phases on labels in global memory,
  * eight members interleaved per 32-byte sector, and EDGES and SAMPLED run one

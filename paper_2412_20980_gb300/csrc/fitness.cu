@@ -794,14 +794,16 @@ int gapa_launch_read_probe(const void* buf, size_t bytes, int passes, int grid, 
 bool gapa_fitness_local(const gapa_ctx* c) {
     const DeviceGraph& g = c->g;
     // AUTO: not where most deletions leave much apart (mean degree below 3: trees, sparse random graphs), and on
-    // graphs of up to 2048 nodes only from a mean degree of 5.75 and 5700 arcs on.  Cut-local time against the
+    // graphs of up to 2048 nodes only from a mean degree of 5.75 on, with 5700 arcs or, where the largest degree is
+    // eight times the mean (short chains of phases on random members), 650 nodes.  Cut-local time against the
     // full pipeline's, least to most over 100 and 1000 members of n / 50 to n / 8 genes, random and hub-heavy:
     // n = 300, degree 4 to 8: 0.71 to 1.95, 16: 0.59 to 0.89; n = 500, degree 6: 0.84 to 1.37, 10 to 12: 0.71 to 1.16;
-    // n = 700, degree 6: 0.76 to 1.40, 8: 0.75 to 1.32, 10 to 12: 0.60 to 1.00; n = 1000, degree 4 to 5.5: 0.94 to 1.45,
+    // n = 700, degree 6: BA and HK 0.76 to 1.13, G(n, M) 1.02 to 1.40, 8: 0.75 to 1.07 and 0.88 to 1.32, 10 to 12: 0.60 to 1.00; n = 1000, degree 4 to 5.5: 0.94 to 1.45,
     // 6 (BA, HK, G(n, M)): 0.63 to 1.13, 8: 0.57 to 1.12; n = 1400, degree 6: 0.51 to 1.01.  Above 2048 nodes it takes over
     // from a kernel that it is faster than at every degree (0.65 of its time on average, lattices and community
     // graphs among them, where single calls take up to 1.8 times as long).
-    const bool small = g.n <= 2048 && (g.mean_deg_x16 < 92 || g.nnz < 5700);
+    const bool tail = 16ll * g.max_degree >= 8ll * g.mean_deg_x16;
+    const bool small = g.n <= 2048 && (g.mean_deg_x16 < 92 || (g.nnz < 5700 && !(tail && g.n >= 650)));
     const bool sparse = g.mean_deg_x16 < 48 || small;
     return g.packed16 && g.lc.par && (c->fitness_variant == GAPA_FITNESS_TREE_LOCAL ||
                                       (c->fitness_variant == GAPA_FITNESS_AUTO && !sparse));

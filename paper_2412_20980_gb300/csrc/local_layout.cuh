@@ -23,9 +23,12 @@ GAPA_LAYOUT_FN size_t tree32_smem_bytes(int n) { return (size_t)n * 4 + (size_t)
 // Layout of one member of the cut-local kernel: labels (16-byte units for the bulk copy), the list
 // region (16-bit node ids, then the bitmap of listed nodes), twelve team scalars and the mbarrier.
 GAPA_LAYOUT_FN size_t tree16l_bitmap_bytes(int n) { return ((((size_t)n + 31) >> 5) * 4 + 15) & ~(size_t)15; }
-// The tops beyond which a member runs the full pipeline on 32-bit labels, by 16 times the mean degree.
+// The tops beyond which a member runs the full pipeline on 32-bit labels, by 16 times the mean degree.  Measured
+// on BA, HK and G(n, M) graphs of mean degree 4 (2500 to 52000 nodes, 40 to 1000 members), n / 16, n / 8, n / 5 and
+// n / 3: random sets 0.68, 0.56, 0.53 and 0.53 of the former kernel's time, hub-heavy ones 0.86, 0.77, 0.74 and 0.76 (at
+// most 1.28, 1.17, 1.16 and 1.74).
 GAPA_LAYOUT_FN bool tree16l_sparse(int mean_deg_x16) { return mean_deg_x16 < 80; }
-GAPA_LAYOUT_FN int tree16l_tops_max(int n, int mean_deg_x16) { return tree16l_sparse(mean_deg_x16) ? n / 8 : n; }
+GAPA_LAYOUT_FN int tree16l_tops_max(int n, int mean_deg_x16) { return tree16l_sparse(mean_deg_x16) ? n / 5 : n; }
 // The least list region: the full pipeline's bitmap and scalars, and 512 entries (sparse graphs: all of
 // the full pipeline on 32-bit labels).
 GAPA_LAYOUT_FN size_t tree16l_min_list_bytes(int n, int mean_deg_x16) {

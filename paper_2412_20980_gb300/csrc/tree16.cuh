@@ -738,10 +738,11 @@ __device__ __forceinline__ int tree16l_owner(const int* off, int owners, int i) 
 // graphs with an eighth of the nodes deleted, up to all of them hubs, 0.16 n on
 // G(n, M) of mean degree 3; small-world and community graphs lose 2 to 3
 // members of 40 there.  Half of the graph as the limit made these 1.2 to 1.5
-// times slower, a look at the share apart half-way through 1.3 to 1.9.)  On sparse graphs (mean degree below 5) a member with more
-// than n / 8 tops, which leaves thousands of nodes apart, runs tree32_member
-// from the start (2 links per node, n = 12000, 100 hub-heavy members of 600
-// genes: 107 us without).
+// times slower, a look at the share apart half-way through 1.3 to 1.9.)  On
+// sparse graphs (mean degree below 5) a member with more than n / 5 tops, which
+// leaves thousands of nodes apart, runs tree32_member from the start (2 links
+// per node, n = 12000, 100 hub-heavy members of 600 genes: 107 us without;
+// local_layout.cuh has other shares).
 //
 // What bounds it: instruction issue and shared-memory reads (68 % and 30 % of
 // peak on hub-heavy members), and the chain of about ten short phases between

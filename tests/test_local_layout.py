@@ -33,7 +33,7 @@ extern "C" int check(int top, int deg16, int s, int sms, size_t per_sm, size_t r
               : x.threads % 32 || x.threads < 32 || x.threads > 1024 || x.threads * x.per_sm > 2048 ? 5
               // the fallbacks' own extents: bitmap and four scalars, or 32-bit labels, bitmap and scalars
               : (size_t)((n + 31) / 32) * 4 + 16 > list ? 6
-              : n / 8 >= 1 && tree16l_tops_max(n, deg16) < n && tree32_smem_bytes(n) > tree16_lab_bytes(n) + list ? 7 : 0;
+              : tree16l_tops_max(n, deg16) < n && tree32_smem_bytes(n) > tree16_lab_bytes(n) + list ? 7 : 0;
         if (*rule) return n;
     }
     return 0;
@@ -65,7 +65,7 @@ def test_layout_holds_every_fallback(layout, deg16, static):
         assert n == 0, f"n = {n}, s = {s}: rule {rule.value}"
 
 
-# sets of more than n / 8 tops, which a graph of two links per node hands to the 32-bit pipeline, at the
+# sets of more than n / 5 tops, which a graph of two links per node hands to the 32-bit pipeline, at the
 # largest sizes of the kernel and past them
 @pytest.mark.gpu
 @pytest.mark.parametrize("n", [56083, 56084, 56099, 56265, 56284])
@@ -81,7 +81,7 @@ def test_largest_graphs_match_oracle(layout, n):
     order = np.argsort(-g.degrees(), kind="stable").astype(np.int32)
     k, s = n // 6, 160
     pop = np.stack([rng.permutation(n)[:k] for _ in range(s)]).astype(np.int32)
-    for i in range(0, s, 2):  # half of the genes among the hubs, so far more tops than n / 8
+    for i in range(0, s, 2):  # half of the genes among the hubs, so more tops than n / 5
         rest = order[k // 2:]
         pop[i] = np.concatenate([order[:k // 2], rest[rng.permutation(rest.size)[:k - k // 2]]])
     pop[3, 1] = pop[3, 0]  # a repeated gene: the 16-bit pipeline
@@ -100,7 +100,7 @@ def test_largest_graphs_match_oracle(layout, n):
 # by the launches of a call that does not fit the SMs at once: the full pipeline is one, the cut-local kernel
 # comes after its cost estimates and order
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,edges,launches", [(300, 1800, 1), (950, 2849, 1), (1000, 2850, 3), (500, 2850, 3),
+@pytest.mark.parametrize("n,edges,launches", [(649, "ba", 1), (650, "ba", 3), (300, 1800, 1), (950, 2849, 1), (1000, 2850, 3), (500, 2850, 3),
                                               (2000, 5600, 1), (2048, 5888, 3), (2049, 3074, 3), (2049, 3009, 1)])
 def test_automatic_choice_on_both_sides_of_its_lines(n, edges, launches):
     import torch
@@ -108,7 +108,7 @@ def test_automatic_choice_on_both_sides_of_its_lines(n, edges, launches):
     from paper_2412_20980_gb300 import Context, build
 
     build.build()
-    g = synth.er_graph(n, edges, 7)
+    g = synth.ba_graph(n, 4, 1) if edges == "ba" else synth.er_graph(n, edges, 7)
     s = 9 * torch.cuda.get_device_properties(0).multi_processor_count
     pop = synth.random_deletion_sets(n, n // 20, s, 5)
     with Context(0) as ctx:
