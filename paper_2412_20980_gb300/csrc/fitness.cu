@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(1024) cc_smem_kernel(GraphArgs g, const int* _
     member_pc<kVar>(smem_lab, g, pop + (size_t)i * k, k, &fit[i], status, red, &sh_root);
 }
 
-// The cut-local kernel, at most 32 registers per thread: 2048 threads per SM.
+// The cut-local kernel, at most 32 registers per thread (none spilled): 2048 threads per SM.
 __global__ void __launch_bounds__(1024, 2) cc_local_kernel(const __grid_constant__ GraphArgs g,
                                                            const int* __restrict__ pop, int k,
                                                            long long* __restrict__ fit, int* status,
@@ -593,7 +593,7 @@ int check_shape(const gapa_ctx* c, const gapa_dev::LocalShape& shape) {
 }
 
 // The cut-local kernel: members costliest first where not all of them run at once (estimates precomputed by
-// the operator kernel, or here; in order, the calls above take 70 and 97 us).
+// the operator kernel, or here; in order, the two calls measured at local_shape take 70 and 97 us).
 int launch_local(gapa_ctx* c, const GraphArgs& ga, const int32_t* pop, int s, int k, long long* f, cudaStream_t st,
                  int* kernels, const unsigned* est_in) {
     const gapa_dev::LocalShape shape = local_shape(c, s);

@@ -744,8 +744,8 @@ __device__ __forceinline__ int tree16l_owner(const int* off, int owners, int i) 
 // per node, n = 12000, 100 hub-heavy members of 600 genes: 107 us without;
 // local_layout.cuh has other shares).
 //
-// What bounds it: instruction issue and shared-memory reads (68 % and 30 % of
-// peak on hub-heavy members), and the chain of about ten short phases between
+// What bounds it: instruction issue and shared-memory reads (55 % and 43 % of
+// peak on hub-heavy members, 45 % and 31 % on random ones), and the chain of about ten short phases between
 // team barriers, each one or two L2 reads deep; so members in flight per SM
 // count most, which 16-bit labels serve.  Measured, 1023 members of 1000 genes
 // at n = 20000 (kernel): random 86 us before (32-bit labels, listing down the
