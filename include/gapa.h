@@ -293,7 +293,7 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * TREE_LOCAL reaches the same components with work local to the deletion: the
  * tree parents are bulk-copied into the labels, the children of deleted nodes
  * take a live lower-numbered neighbour (or are united with higher-numbered
- * ones), and only the classes left apart from the first live node's are listed
+ * ones), and only the classes left apart from one reference root's are listed
  * and searched; a member with repeated genes, or whose lists outgrow the
  * kernel's shared memory, takes the TREE path.  It needs a graph whose 16-bit
  * ids and labels fit in shared memory (n up to 56,281 on GB300).
@@ -322,7 +322,10 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * (a union of two pieces), and only the nodes outside the largest resulting
  * class scan their arcs.  Members estimated to list over a quarter of the
  * nodes, or beyond the kernel's shared-memory capacities, run the TREE_LOCAL
- * kernel instead.  Same graphs as TREE_LOCAL; PC and MCN objectives. */
+ * kernel instead.  Same graphs as TREE_LOCAL; PC and MCN objectives.  Its
+ * tables are made when it is chosen, or by the upload after that
+ * (GAPA_ERR_OOM if they do not fit; not while the stream is captured, when
+ * the TREE setting runs). */
 #define GAPA_FITNESS_PIECE 7
 /* SPARSE (AUTO's choice where the labels do not fit in shared memory, and
  * selectable on any graph): work proportional to what the deletion disturbs.
@@ -339,8 +342,11 @@ int gapa_run_surrogate(gapa_ctx* ctx, const gapa_config* cfg, gapa_surrogate* sg
  * CTA per member with the deletion bitmap, the deleted nodes and their child
  * offsets in shared memory (n/8 + 8k bytes + 12 KB: n = 2^20 with k up to
  * about 12,000 on GB300; otherwise the TREE setting runs), per-CTA state in
- * library-owned global scratch (32 bytes per node per resident CTA), cleared
- * after each member.  PC and MCN objectives. */
+ * library-owned global scratch (24 bytes per node and 20 per component of two
+ * nodes or more, per resident CTA), cleared after each member.  Large
+ * populations of light members on graphs of mean degree 3.5 and more run two
+ * or six smaller CTAs per SM, where the scratch can be had.  PC and MCN
+ * objectives. */
 #define GAPA_FITNESS_SPARSE 8
 int gapa_set_fitness_kernel(gapa_ctx* ctx, int variant);
 
